@@ -124,7 +124,7 @@ int split_exp(const corr* h) {
     return e;
 }
 
-// frames per TMEM accumulation chunk of CORR_FP32TC: 128, and 256 where the X-engine pairs the
+// frames per TMEM accumulation chunk of CORR_FP32TC: 128, and 512 where the X-engine pairs the
 // hi and lo rows (64 inputs), whose drain then adds two accumulator halves per chunk
 constexpr int kSplitChunk = 128;
 constexpr int kSplitChunkPaired = 512;
@@ -220,7 +220,7 @@ int gbx::run_integration(corr* h, const int8_t* x, int64_t ld, int64_t n_avail, 
         CU(launch_xengine_fp32(xp, h->n_sm, s));
     else
         CU(launch_xengine_tc_table(h->out_buf == 1 ? h->xtab_b1 : h->d_xtab, h->n_items, h->n_sm, s,
-                                   h->xmode == CORR_FP32TC ? XT_FORM_F32 : fmode == OUT_I8B ? XT_FORM_I8 : XT_FORM_F16));
+                                   h->xmode == CORR_FP32TC ? xt_form_f32(h->n_in) : fmode == OUT_I8B ? XT_FORM_I8 : XT_FORM_F16));
     if (h->dump > 0) {
         CU(launch_power_dumps(static_cast<const float*>(h->d_spec), h->n_in, h->n_chan, h->n_int, h->dump,
                               h->d_power, s, fmode == OUT_F32Q));

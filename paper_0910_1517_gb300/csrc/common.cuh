@@ -72,6 +72,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsign
     return true;
 }
 
+// The same wait for a whole converged warp, with one answer for it: every lane tests the barrier and
+// the vote decides.  (One lane polling behind a branch and a shuffle of its answer took about 300
+// cycles a call in the X-engine's converters even with the barrier complete, this about 120.)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, unsigned* err, unsigned bit) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+        if (__any_sync(0xffffffffu, clock64() - t0 > kWaitBudgetCycles)) {
+            if (err && (threadIdx.x & 31) == 0) atomicOr(err, bit);
+            return false;
+        }
+    }
+    return true;
+}
+
 // 1-D bulk copy global -> shared through the TMA engine, completing on `bar`.
 // dst, src 16-byte aligned; bytes a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -126,6 +141,15 @@ __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+
+// True in one lane of a converged warp, the same lane every time.  The compiler knows that a single
+// lane runs the branch, so that tcgen05 operands computed from warp-uniform values stay in uniform
+// registers.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
 }
 
 // Arrive on `bar` once every tcgen05.mma issued so far by this thread has completed.
@@ -280,6 +304,15 @@ __device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&v)[8]) {
                  "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
 }
+
+// ------------------------------------------------------------- register split
+
+// Registers a thread of this warpgroup from here on (all its warps): the increases wait until the
+// block's other warpgroups have given up theirs, so the shares must add up to the launch's at most.
+template <int N_REG>
+__device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N_REG)); }
+template <int N_REG>
+__device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N_REG)); }
 
 // ------------------------------------------------------------- complex math
 

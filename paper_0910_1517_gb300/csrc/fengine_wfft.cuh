@@ -85,11 +85,6 @@ struct WCtl {
     int Ds[kMaxAnt];
 };
 
-template <int N_REG>
-__device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N_REG)); }
-template <int N_REG>
-__device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N_REG)); }
-
 template <int M, int MODE>
 __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams p) {
     using P = WPlan<M>;

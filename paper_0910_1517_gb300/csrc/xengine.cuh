@@ -73,10 +73,11 @@ bool xengine_tc_encode_quad(XtSub& x);
 bool xengine_tc_supported(int n_in);                 // 2 n_in <= 256
 int xengine_tc_max_ks(int n_in);                      // largest fp16 stage for the row count
 int xengine_tc_ks_fp32(int n_in);                     // largest FP32-form stage (FP32 slot <= kStage2Bytes)
-size_t xengine_tc_smem();
 // form of every sub-array of the table: one fp16 plane (XT_FORM_F16), FP32 split on chip (spec32,
-// XT_FORM_F32) or int8 bytes widened on chip (in8, XT_FORM_I8)
-enum XtForm : int { XT_FORM_F16 = 0, XT_FORM_F32 = 1, XT_FORM_I8 = 2 };
+// XT_FORM_F32, or XT_FORM_F32P when every sub-array has 64 inputs) or int8 bytes widened on chip
+// (in8, XT_FORM_I8)
+enum XtForm : int { XT_FORM_F16 = 0, XT_FORM_F32 = 1, XT_FORM_I8 = 2, XT_FORM_F32P = 3 };
+constexpr XtForm xt_form_f32(int n_in) { return 2 * n_in == 128 ? XT_FORM_F32P : XT_FORM_F32; }
 cudaError_t launch_xengine_tc_table(const XtBatch* dtab, int n_items, int n_sm, cudaStream_t s, int form = XT_FORM_F16);
 
 }  // namespace gbx
