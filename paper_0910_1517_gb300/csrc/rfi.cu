@@ -1,6 +1,7 @@
 // rfi.cu -- RFI-flagging stage for sm_103a: per-patch median / MAD statistics and
 // flags (Sec. 5, Eq. 3-4), and a small convolutional flagger trained and run by
-// hand-written kernels (direct 3x3 convolutions over 16x16 output tiles, FP16
+// hand-written kernels (the FP16 flagger's forward pass is rfi_tc.cu's; the rest
+// here are direct 3x3 convolutions over 16x16 output tiles, FP16
 // weights and activations, FP32 accumulation, FP32 gradients, Adam on FP32
 // master weights).  Every network kernel is templated on the type TA its weights
 // and activations are kept in: __half for the flagger, float for the FP32 build
@@ -16,6 +17,7 @@
 #include "../../include/corr.h"
 #include "../../include/rfi.h"
 #include "common.cuh"
+#include "rfi_tc.cuh"
 
 namespace gbx {
 void set_last_error(const char* msg);
@@ -244,6 +246,7 @@ struct Wts {
     TA* pf16;                   // [NPAR] flat
     TA *wf1, *wf2, *wf3;        // forward  [CI][9][CO]
     TA *wb3, *wb2;              // backward [CO_fwd][9][CI_fwd], taps flipped
+    unsigned char* pack;        // fp16: the tensor-core forward pass's operands (rfi_pack1 .. 3)
 };
 
 template <typename TA>
@@ -269,6 +272,9 @@ __global__ void transform_kernel(const float* __restrict__ p, Wts<TA> w) {
         c = (off / 9) % ci;
         tap = off % 9;
         fwd[(c * 9 + tap) * co + o] = h;                         // [c][tap][o]
+        if constexpr (sizeof(TA) == 2) {
+            if (ci > 1) *reinterpret_cast<TA*>(w.pack + (ci == 16 ? gbx::rfi_pack2(o, c, tap) : gbx::rfi_pack3(o, c, tap))) = h;
+        }
         if (bwd) bwd[(o * 9 + (8 - tap)) * ci + c] = h;          // [o][8 - tap][c]
     }
 }
@@ -354,7 +360,8 @@ struct rfi_net {
     int step = 0;
     int fp32 = 0;                        // weights and activations in FP32 (rfi_create_fp32), else FP16
     float *p = nullptr, *m = nullptr, *v = nullptr, *g = nullptr, *loss = nullptr;
-    void* w[6] = {};                     // Wts<TA>: pf16, wf1, wf2, wf3, wb3, wb2
+    void* w[7] = {};                     // Wts<TA>: pf16, wf1, wf2, wf3, wb3, wb2, pack
+    unsigned* err = nullptr;             // device error word of the tensor-core kernel's bounded waits
     void *A1 = nullptr, *A2 = nullptr, *A3 = nullptr;   // TA activations
     float *dA1 = nullptr, *dA2 = nullptr, *dA3 = nullptr;
     int n_sm = 0;
@@ -384,6 +391,7 @@ Wts<TA> wts(rfi_net* n) {
     w.wf3 = static_cast<TA*>(n->w[3]);
     w.wb3 = static_cast<TA*>(n->w[4]);
     w.wb2 = static_cast<TA*>(n->w[5]);
+    w.pack = static_cast<unsigned char*>(n->w[6]);
     return w;
 }
 
@@ -420,11 +428,41 @@ int forward_t(rfi_net* n, const uint16_t* x, int B, cudaStream_t s) {
     return CORR_OK;
 }
 
+// The FP16 flagger's forward pass on the tensor cores: probabilities and / or the activations a
+// backward pass reads (keep)
+int forward_tc(rfi_net* n, const uint16_t* x, int B, float* prob, bool keep, cudaStream_t s) {
+    const Wts<__half> w = wts<__half>(n);
+    gbx::RfiFwd f{};
+    f.x = reinterpret_cast<const __half*>(x);
+    f.pack = w.pack;
+    f.w1 = w.pf16 + OW1;
+    f.b1 = w.pf16 + OB1;
+    f.b2 = w.pf16 + OB2;
+    f.b3 = w.pf16 + OB3;
+    f.w4 = w.pf16 + OW4;
+    f.b4 = w.pf16 + OB4;
+    f.prob = prob;
+    if (keep) {
+        f.A1 = static_cast<__half*>(n->A1);
+        f.A2 = static_cast<__half*>(n->A2);
+        f.A3 = static_cast<__half*>(n->A3);
+    }
+    f.B = B;
+    f.err = n->err;
+    RCU(gbx::launch_rfi_forward_tc(f, n->n_sm, s));
+    return CORR_OK;
+}
+
 template <typename TA>
 int forward_backward_t(rfi_net* n, const uint16_t* x, const uint8_t* mask, int B, cudaStream_t s) {
     RCU(cudaMemsetAsync(n->g, 0, sizeof(float) * NPAR, s));
     RCU(cudaMemsetAsync(n->loss, 0, sizeof(float), s));
-    if (int rc = forward_t<TA>(n, x, B, s)) return rc;
+    if constexpr (sizeof(TA) == 2) {
+        // 16-byte loads of the patches: any other alignment takes the CUDA-core layers
+        if (int rc = reinterpret_cast<uintptr_t>(x) & 15 ? forward_t<TA>(n, x, B, s) : forward_tc(n, x, B, nullptr, true, s)) return rc;
+    } else {
+        if (int rc = forward_t<TA>(n, x, B, s)) return rc;
+    }
     const Wts<TA> w = wts<TA>(n);
     TA *A1 = static_cast<TA*>(n->A1), *A2 = static_cast<TA*>(n->A2), *A3 = static_cast<TA*>(n->A3);
     const int64_t npx = static_cast<int64_t>(B) * PHW;
@@ -438,10 +476,6 @@ int forward_backward_t(rfi_net* n, const uint16_t* x, const uint8_t* mask, int B
     RCU((wgrad<1, 16, __half, TA>(reinterpret_cast<const __half*>(x), n->dA1, A1, n->g + OW1, n->g + OB1, B,
                                   n->n_sm, s)));
     return CORR_OK;
-}
-
-int forward(rfi_net* n, const uint16_t* x, int B, cudaStream_t s) {
-    return n->fp32 ? forward_t<float>(n, x, B, s) : forward_t<__half>(n, x, B, s);
 }
 
 int forward_backward(rfi_net* n, const uint16_t* x, const uint8_t* mask, int B, cudaStream_t s) {
@@ -468,6 +502,15 @@ int head_infer(rfi_net* n, int B, float* prob, cudaStream_t s) {
                                                  0.0f, nullptr, nullptr, nullptr, prob);
     RCU(cudaGetLastError());
     return CORR_OK;
+}
+
+// After a synchronisation: a bounded wait of the tensor-core kernel ran out since the last check
+int check_err(rfi_net* n) {
+    unsigned err = 0;
+    RCU(cudaMemcpy(&err, n->err, sizeof err, cudaMemcpyDeviceToHost));
+    if (!err) return CORR_OK;
+    RCU(cudaMemset(n->err, 0, sizeof err));
+    return rfail(CORR_E_TIMEOUT, "a kernel wait of the flagger timed out; results since the last synchronous call are invalid");
 }
 
 int check_batch(rfi_net* n, const void* x, int B) {
@@ -499,6 +542,9 @@ int create(rfi_net_t** out, int max_batch, int fp32) {
     const size_t wn[6] = {NPAR, 144, 4608, 4608, 4608, 4608};
     for (int q = 0; q < 6; ++q)
         if (e == cudaSuccess) e = cudaMalloc(&n->w[q], ta * wn[q]);
+    if (e == cudaSuccess) e = cudaMalloc(&n->w[6], gbx::kRfiPackBytes);
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&n->err), sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMemset(n->err, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc(&n->A1, ta * px * 16);
     if (e == cudaSuccess) e = cudaMalloc(&n->A2, ta * px * 32);
     if (e == cudaSuccess) e = cudaMalloc(&n->A3, ta * px * 16);
@@ -527,7 +573,7 @@ int rfi_create_fp32(rfi_net_t** out, int max_batch) { return create(out, max_bat
 int rfi_destroy(rfi_net_t* n) {
     if (!n) return CORR_OK;
     void* bufs[] = {n->p, n->m, n->v, n->g, n->loss, n->w[0], n->w[1], n->w[2], n->w[3], n->w[4],
-                    n->w[5], n->A1, n->A2, n->A3, n->dA1, n->dA2, n->dA3};
+                    n->w[5], n->w[6], n->err, n->A1, n->A2, n->A3, n->dA1, n->dA2, n->dA3};
     for (void* b : bufs)
         if (b) cudaFree(b);
     delete n;
@@ -551,7 +597,7 @@ int rfi_get_params(rfi_net_t* n, float* params) {
     if (!n || !params) return rfail(CORR_E_INVAL, "rfi_get_params: null argument");
     RCU(cudaDeviceSynchronize());
     RCU(cudaMemcpy(params, n->p, sizeof(float) * NPAR, cudaMemcpyDeviceToHost));
-    return CORR_OK;
+    return check_err(n);
 }
 
 int rfi_loss_grad(rfi_net_t* n, const uint16_t* x, const uint8_t* mask, int B, float* loss, float* grad,
@@ -564,7 +610,7 @@ int rfi_loss_grad(rfi_net_t* n, const uint16_t* x, const uint8_t* mask, int B, f
     RCU(cudaMemcpy(loss, n->loss, sizeof(float), cudaMemcpyDeviceToHost));
     *loss /= static_cast<float>(static_cast<int64_t>(B) * PHW);
     if (grad) RCU(cudaMemcpy(grad, n->g, sizeof(float) * NPAR, cudaMemcpyDeviceToHost));
-    return CORR_OK;
+    return check_err(n);
 }
 
 int rfi_train_step(rfi_net_t* n, const uint16_t* x, const uint8_t* mask, int B, float lr, float* loss,
@@ -582,6 +628,7 @@ int rfi_train_step(rfi_net_t* n, const uint16_t* x, const uint8_t* mask, int B, 
         RCU(cudaStreamSynchronize(s));
         RCU(cudaMemcpy(loss, n->loss, sizeof(float), cudaMemcpyDeviceToHost));
         *loss /= static_cast<float>(static_cast<int64_t>(B) * PHW);
+        return check_err(n);
     }
     return CORR_OK;
 }
@@ -590,7 +637,8 @@ int rfi_infer(rfi_net_t* n, const uint16_t* x, int B, float* prob, void* stream)
     if (int rc = check_batch(n, x, B)) return rc;
     if (!prob) return rfail(CORR_E_INVAL, "rfi_infer: prob is null");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (int rc = forward(n, x, B, s)) return rc;
+    if (!n->fp32 && !(reinterpret_cast<uintptr_t>(x) & 15)) return forward_tc(n, x, B, prob, false, s);
+    if (int rc = n->fp32 ? forward_t<float>(n, x, B, s) : forward_t<__half>(n, x, B, s)) return rc;
     return head_infer(n, B, prob, s);
 }
 
