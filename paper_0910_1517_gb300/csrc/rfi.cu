@@ -293,59 +293,99 @@ __global__ void adam_kernel(float* __restrict__ p, float* __restrict__ m, float*
 }
 
 // ------------------------------------------------------------ patch stats
-// One CTA per patch: gather its 4096 powers, bitonic-sort a copy for the median, sort the
-// absolute deviations for the MAD, then write Eq. 4 flags and the compressed network input.
-__device__ void bitonic4096(float* s) {
-    for (int k = 2; k <= PHW; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < PHW; i += blockDim.x) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const float a = s[i], b = s[l];
-                    const bool up = (i & k) == 0;
-                    if ((a > b) == up) {
-                        s[i] = b;
-                        s[l] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+// A warp takes a patch: its 4096 powers in registers (lane: two columns of each of the 64 rows), the
+// two middle ranks of the powers and of the absolute deviations by bisection over the bit patterns
+// of the floats between their extremes -- count the values at or below the middle one, some 25 to
+// 31 times -- then the Eq. 4 flags and the compressed network input.  No shared memory, no barrier.
+// What bounds it: the counting, about 2 instructions a value and step.  4096 patches: 0.17 ms; 1.44 ms
+// with two bitonic sorts of the patch in shared memory (78 barriers each).
+
+// the floats in the order of their values as unsigned integers, and back
+__device__ __forceinline__ uint32_t key_of(float f) {
+    const uint32_t u = __float_as_uint(f);
+    return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float of_key(uint32_t k) { return __uint_as_float(k & 0x80000000u ? k & 0x7fffffffu : ~k); }
+
+// Mean of the two middle values of the warp's 4096 values get(q), q < 128 a lane (NaN sorts last).
+template <typename Get>
+__device__ __forceinline__ float median4096(const Get& get) {
+    constexpr int kPer = PHW / 32;
+    float mn = INFINITY, mx = -INFINITY;                   // (fminf and fmaxf pass NaN over)
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        mn = fminf(mn, get(q));
+        mx = fmaxf(mx, get(q));
+    }
+    uint32_t lo = __reduce_min_sync(0xffffffffu, key_of(mn)), hi = __reduce_max_sync(0xffffffffu, key_of(mx));
+    auto at_or_below = [&](float t) {
+        int n = 0;
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) n += get(q) <= t;
+        return __reduce_add_sync(0xffffffffu, n);
+    };
+    while (lo < hi) {                                      // the smallest value with 2048 at or below it
+        const uint32_t mid = lo + (hi - lo) / 2;
+        if (at_or_below(of_key(mid)) >= PHW / 2) hi = mid;
+        else lo = mid + 1;
+    }
+    const float a = of_key(lo);
+    if (at_or_below(a) > PHW / 2) return 0.5f * (a + a);
+    float next = INFINITY;                                 // the next larger one
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) next = get(q) > a ? fminf(next, get(q)) : next;
+    return 0.5f * (a + of_key(__reduce_min_sync(0xffffffffu, key_of(next))));
 }
 
-__global__ void __launch_bounds__(1024) patch_kernel(const float* __restrict__ P, int n_dump, int n_chan, float M,
-                                                     __half* __restrict__ x, uint8_t* __restrict__ flags,
-                                                     float* __restrict__ stats) {
-    __shared__ float v[PHW];
-    __shared__ float s[PHW];
-    const int nkw = n_chan / PW, ndw = n_dump / PH;
-    const int b = blockIdx.x;
+__global__ void __launch_bounds__(128, 3) patch_kernel(const float* __restrict__ P, int B, int n_dump, int n_chan, float M,
+                                                       __half* __restrict__ x, uint8_t* __restrict__ flags,
+                                                       float* __restrict__ stats) {
+    const int nkw = n_chan / PW, ndw = n_dump / PH, lane = threadIdx.x % 32;
+    const int b = blockIdx.x * 4 + threadIdx.x / 32;
+    if (b >= B) return;
     const int kw = b % nkw, dw = (b / nkw) % ndw, i = b / (nkw * ndw);
-    for (int q = threadIdx.x; q < PHW; q += blockDim.x) {
-        const int h = q / PW, w = q % PW;
-        const float val = P[(static_cast<int64_t>(i) * n_dump + dw * PH + h) * n_chan + kw * PW + w];
-        v[q] = val;
-        s[q] = val;
+    const float* src = P + (static_cast<int64_t>(i) * n_dump + dw * PH) * n_chan + kw * PW + 2 * lane;
+    const bool wide = !(reinterpret_cast<uintptr_t>(P) & 7);   // rows are multiples of 256 bytes: the base decides
+    auto row = [&](int h) {
+        const float* r = src + static_cast<int64_t>(h) * n_chan;
+        return wide ? __ldg(reinterpret_cast<const float2*>(r)) : make_float2(__ldg(r), __ldg(r + 1));
+    };
+    float v[PHW / 32];
+#pragma unroll
+    for (int h = 0; h < PH; ++h) {
+        const float2 t = row(h);
+        v[2 * h] = t.x;
+        v[2 * h + 1] = t.y;
     }
-    __syncthreads();
-    bitonic4096(s);
-    const float med = 0.5f * (s[PHW / 2 - 1] + s[PHW / 2]);
-    __syncthreads();
-    for (int q = threadIdx.x; q < PHW; q += blockDim.x) s[q] = fabsf(v[q] - med);
-    __syncthreads();
-    bitonic4096(s);
-    const float mad = 0.5f * (s[PHW / 2 - 1] + s[PHW / 2]);
-    const float sig = mad / 0.6745f;
-    for (int q = threadIdx.x; q < PHW; q += blockDim.x) {
-        const float dev = v[q] - med;
-        const int64_t o = static_cast<int64_t>(b) * PHW + q;
-        if (flags) flags[o] = fabsf(dev) > M * sig ? 1 : 0;
-        if (x) {
-            const float u = sig > 0.0f ? dev / sig : 0.0f;
-            x[o] = __float2half_rn(copysignf(log1pf(fabsf(u)), u));
+    const float med = median4096([&](int q) { return v[q]; });
+    const float mad = median4096([&](int q) { return fabsf(v[q] - med); });
+    const float sig = mad / 0.6745f, thr = M * sig;
+    const bool pair = !((reinterpret_cast<uintptr_t>(x) & 3) | (reinterpret_cast<uintptr_t>(flags) & 1));
+#pragma unroll 4
+    for (int h = 0; h < PH; ++h) {                          // (read again: from the registers it would have to be unrolled)
+        const int64_t o = static_cast<int64_t>(b) * PHW + h * PW + 2 * lane;
+        const float2 t = row(h);
+        float u[2];
+        uint8_t f[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float dev = (e ? t.y : t.x) - med;
+            f[e] = fabsf(dev) > thr ? 1 : 0;
+            const float r = sig > 0.0f ? dev / sig : 0.0f;
+            u[e] = x ? copysignf(log1pf(fabsf(r)), r) : 0.0f;
+        }
+        if (pair) {
+            if (flags) *reinterpret_cast<uchar2*>(flags + o) = make_uchar2(f[0], f[1]);
+            if (x) *reinterpret_cast<__half2*>(x + o) = __floats2half2_rn(u[0], u[1]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (flags) flags[o + e] = f[e];
+                if (x) x[o + e] = __float2half_rn(u[e]);
+            }
         }
     }
-    if (stats && threadIdx.x == 0) {
+    if (stats && lane == 0) {
         stats[2 * b] = med;
         stats[2 * b + 1] = mad;
     }
@@ -647,8 +687,8 @@ int rfi_patches(const float* power, int n_in, int n_dump, int n_chan, float M, u
     if (!power || n_in < 1 || n_dump < PH || n_chan < PW || n_dump % PH || n_chan % PW || !(M > 0.0f))
         return rfail(CORR_E_INVAL, "rfi_patches: need n_dump, n_chan multiples of 64 and M > 0");
     const int B = n_in * (n_dump / PH) * (n_chan / PW);
-    patch_kernel<<<B, 1024, 0, static_cast<cudaStream_t>(stream)>>>(power, n_dump, n_chan, M,
-                                                                    reinterpret_cast<__half*>(x), mad_flags, stats);
+    patch_kernel<<<(B + 3) / 4, 128, 0, static_cast<cudaStream_t>(stream)>>>(power, B, n_dump, n_chan, M,
+                                                                             reinterpret_cast<__half*>(x), mad_flags, stats);
     RCU(cudaGetLastError());
     return CORR_OK;
 }
