@@ -14,11 +14,11 @@
 //
 // Rounding.  The tensor core adds the products of an output in another order than the CUDA-core
 // kernels; where the FP32 sum lies next to a rounding boundary of fp16 the activation could round
-// the other way, a whole fp16 step.  Activations of layers 2 and 3 within 16 FP32 steps of a boundary
-// (0.4 % of them) are therefore listed and summed again in FP32 in the CUDA-core order, one a
-// thread: on 4096 patches the probabilities are then within 9.5e-7 (relative 2-norm) of that order's
-// and 1.9e-4 at most, without 1.6e-5 and up to 2.9e-3.  The lists cost 0.15 ms and the sums 0.34 ms
-// of the 1.6 ms.
+// the other way, a whole fp16 step.  Activations of layers 2 and 3 within 64 FP32 steps of a boundary
+// (1.6 % of them) are therefore listed and summed again in FP32 in the CUDA-core order, one a
+// thread: on 4096 patches the probabilities are then within 5e-7 to 9e-7 (relative 2-norm) of that
+// order's and 4e-4 at most; within 16 steps 2.5e-6 and 7.5e-4, 0.2 ms less; with none 1.6e-5 and up
+// to 2.9e-3, 0.7 ms less of the 1.65 ms.
 //
 // Roles: warp 8 issues the MMAs of a layer tile by tile (a commit each), warps 0-7 take the tiles as
 // they complete: bias, ReLU, rounding to fp16, zeros outside the image, and the next layer's
@@ -26,7 +26,7 @@
 //
 // What bounds it: an MMA with N = 16 or 32 takes the tensor core about 40 cycles whatever its N, 144
 // of them a strip (0.6 ms for 4096 patches), and the near ties' sums, one after another by
-// definition, which little runs beside.  4096 patches: 1.6 ms; 10.95 ms with a CUDA-core kernel a
+// definition, which little runs beside.  4096 patches: 1.65 ms; 10.95 ms with a CUDA-core kernel a
 // layer and the head's (conv2 5.0, conv3 5.5, conv1 0.29, head 0.15 ms).  Layer 1's four positions a
 // thread: with one, its weight loads took the pass to 1.97 ms.
 #include <type_traits>
@@ -74,7 +74,7 @@ struct alignas(16) Ctl {
 // r >= 0 within kTieBand FP32 steps of the middle between two fp16 numbers, where rounding turns:
 // the 13 bits that fp16 drops lie around 0x1000 (below fp16's normal numbers and above its largest
 // the answer does not matter)
-constexpr uint32_t kTieBand = 16;
+constexpr uint32_t kTieBand = 64;
 __device__ __forceinline__ bool near_tie(float r) {
     return ((__float_as_uint(r) - (0x1000u - kTieBand)) & 0x1fffu) <= 2 * kTieBand;
 }
@@ -189,10 +189,9 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
     unsigned short* ties = reinterpret_cast<unsigned short*>(smem + Smem::ties);
     // list channels `mask` of position q as near ties of layer 2 (which = 0) or 3
     auto list = [&](uint32_t mask, int q, int which) {
-        for (; mask; mask &= mask - 1) {
-            const int i = atomicAdd(&c.n_tie[which], 1);
+        if (!mask) return;
+        for (int i = atomicAdd(&c.n_tie[which], __popc(mask)); mask; mask &= mask - 1, ++i)
             if (i < kMaxTies) ties[i] = static_cast<unsigned short>(q * 32 + __ffs(mask) - 1);
-        }
     };
     // n channels of pixel (gy, gx), pairs h, to the planar activations A [B][C][64][64]
     auto keep = [&](__half* A, int C, int n, const uint32_t* h, int64_t patch, int gy, int gx) {
