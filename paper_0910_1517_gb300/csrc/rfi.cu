@@ -27,6 +27,16 @@ namespace {
 
 __device__ __forceinline__ float ldf(const __half* p) { return __half2float(*p); }
 __device__ __forceinline__ float ldf(const float* p) { return *p; }
+// four consecutive values; `wide`: the address is aligned to all four
+__device__ __forceinline__ float4 ldf4(const __half* p, bool wide) {
+    if (!wide) return make_float4(ldf(p), ldf(p + 1), ldf(p + 2), ldf(p + 3));
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ float4 ldf4(const float* p, bool wide) {
+    return wide ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+}
 __device__ __forceinline__ void stf(__half* p, float v) { *p = __float2half_rn(v); }
 __device__ __forceinline__ void stf(float* p, float v) { *p = v; }
 
@@ -37,150 +47,227 @@ constexpr int NPAR = 9441;
 constexpr int OW1 = 0, OB1 = 144, OW2 = 160, OB2 = 4768, OW3 = 4800, OB3 = 9408, OW4 = 9424, OB4 = 9440;
 
 // ---------------------------------------------------------------- convolution
-// One CTA computes a 16x16 output tile of one patch for all CO output channels.
-// MODE 0 (forward):       out[o] = relu(b[o] + sum_c sum_tap w[c][tap][o] in[c][pixel + tap])   (fp16 -> fp16)
+// A CTA computes a 16 x 32 output tile of one patch for all CO output channels: a thread takes two
+// rows of four pixels and 8 channels, two channels a packed FP32x2 operation, input channel by input
+// channel and tap by tap (24 window values and 18 16-byte weight reads serve 288 packed operations).
+// MODE 0 (forward):       out[o] = relu(b[o] + sum_c sum_tap w[c][tap][o] in[c][pixel + tap])   (-> TA)
 // MODE 1 (backward data): the same correlation without bias / ReLU on dZ = dA * (act > 0)        (fp32 -> fp32)
-// w is laid out [CI][9][CO] so that one (c, tap) reads CO consecutive weights (a broadcast).
+// w is laid out [CI][9][CO] so that one (c, tap) reads consecutive weights (a broadcast).
 // TIN: type of the forward input (the FP16 patches for layer 1, TA after it); TA: weights and activations.
+// What bounds it: the FP32 pipe, with the shared-memory reads of the weights (four cycles each, shared
+// or not) close behind.  256 patches, backward data of layers 3 / 2: 0.24 / 0.25 ms; 0.33 / 0.43 ms with a
+// pixel a thread (9 or 5 reads for 32 or 16 multiply-adds), no better with four.
+constexpr int CTY = 16, CTX = 32, CPX = 36, CCK = 8;   // tile, row pitch with halo, input channels a round
+constexpr int kCTiles = (PH / CTY) * (PW / CTX);
+
+// dZ of four pixels: the gradients where the activations passed the ReLU
+template <typename TA>
+__device__ __forceinline__ float4 relu_grad4(const float* dA, const TA* act) {
+    const float4 g = ldf4(dA, true), a = ldf4(act, true);
+    return make_float4(a.x > 0.0f ? g.x : 0.0f, a.y > 0.0f ? g.y : 0.0f, a.z > 0.0f ? g.z : 0.0f, a.w > 0.0f ? g.w : 0.0f);
+}
+
+// Rows y0 - 1 .. y0 + ROWS - 2 and columns x0 - 1 .. x0 + COLS of a channel-major image's channels
+// c0 .. c0 + N - 1, zeros outside the patch, to dst[c * CPITCH + row * RPITCH + column].  get4(g) and
+// get1(g) read at index g of the image.
+template <int N, int ROWS, int COLS, int CPITCH, int RPITCH, int NT, typename G4, typename G1>
+__device__ __forceinline__ void load_halo(float* dst, size_t image, int y0, int x0, const G4& get4, const G1& get1) {
+    constexpr int PARTS = COLS / 4;
+    for (int q = threadIdx.x; q < N * ROWS * PARTS; q += NT) {
+        const int part = q % PARTS, yy = (q / PARTS) % ROWS, c = q / (PARTS * ROWS);
+        const int gy = y0 + yy - 1, gx = x0 + 4 * part;
+        const bool in = gy >= 0 && gy < PH;
+        const size_t g = image + static_cast<size_t>(c) * PHW + gy * PW + gx;
+        float* d = dst + c * CPITCH + yy * RPITCH + 4 * part + 1;
+        const float4 v = in ? get4(g) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        d[0] = v.x, d[1] = v.y, d[2] = v.z, d[3] = v.w;
+        if (part == 0) d[-1] = in && gx > 0 ? get1(g - 1) : 0.0f;
+        if (part == PARTS - 1) d[4] = in && gx + 4 < PW ? get1(g + 4) : 0.0f;
+    }
+}
+
 template <int CI, int CO, int MODE, typename TIN, typename TA>
-__global__ void __launch_bounds__(256) conv3x3_kernel(const void* __restrict__ in, const TA* __restrict__ act,
-                                                      const TA* __restrict__ w, const TA* __restrict__ bias,
-                                                      void* __restrict__ out) {
+__global__ void __launch_bounds__(8 * CO) conv3x3_kernel(const void* __restrict__ in, const TA* __restrict__ act,
+                                                         const TA* __restrict__ w, const TA* __restrict__ bias,
+                                                         void* __restrict__ out) {
+    constexpr int CK = CI < CCK ? CI : CCK, NT = 8 * CO, ROWS = CTY + 2;
     extern __shared__ __align__(16) float sm[];
     float* wsm = sm;                                   // CI * 9 * CO
-    float* tile = sm + CI * 9 * CO;                    // CI * TH * TH
-    const int b = blockIdx.x / kTiles, tl = blockIdx.x % kTiles;
-    const int ty0 = (tl / (PW / T)) * T, tx0 = (tl % (PW / T)) * T;
-    const int tid = threadIdx.x, py = tid / T, px = tid % T;
-    for (int q = tid; q < CI * 9 * CO; q += 256) wsm[q] = ldf(w + q);
-    for (int q = tid; q < CI * TH * TH; q += 256) {
-        const int c = q / (TH * TH), r = q % (TH * TH), yy = r / TH, xx = r % TH;
-        const int gy = ty0 + yy - 1, gx = tx0 + xx - 1;
-        float v = 0.0f;
-        if (gy >= 0 && gy < PH && gx >= 0 && gx < PW) {
-            const size_t gi = (static_cast<size_t>(b) * CI + c) * PHW + gy * PW + gx;
-            if constexpr (MODE == 0) {
-                v = ldf(static_cast<const TIN*>(in) + gi);
-            } else {
-                v = static_cast<const float*>(in)[gi];
-                if (!(ldf(act + gi) > 0.0f)) v = 0.0f;             // ReLU gradient
+    float* tile = sm + CI * 9 * CO;                    // CK * ROWS * CPX, column s is pixel s - 1
+    const int b = blockIdx.x / kCTiles, tl = blockIdx.x % kCTiles;
+    const int ty0 = (tl / (PW / CTX)) * CTY, tx0 = (tl % (PW / CTX)) * CTX;
+    const int tid = threadIdx.x, o0 = (tid / 64) * 8, x0 = 4 * (tid % 8), y = 2 * ((tid % 64) / 8);
+    for (int q = tid; q < CI * 9 * CO; q += NT) wsm[q] = ldf(w + q);
+    float2 acc[2][4][4];                               // [row][pixel][channel pair]
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            acc[j / 4][j % 4][e] = MODE == 0 ? make_float2(ldf(bias + o0 + 2 * e), ldf(bias + o0 + 2 * e + 1)) : make_float2(0.0f, 0.0f);
+    const bool wide = (reinterpret_cast<uintptr_t>(in) & 15) == 0;
+    for (int c0 = 0; c0 < CI; c0 += CK) {
+        __syncthreads();                               // the previous round's readers are done
+        const size_t image = (static_cast<size_t>(b) * CI + c0) * PHW;
+        if constexpr (MODE == 0) {
+            const TIN* src = static_cast<const TIN*>(in);
+            load_halo<CK, ROWS, CTX, ROWS * CPX, CPX, NT>(
+                tile, image, ty0, tx0, [&](size_t g) { return ldf4(src + g, wide); }, [&](size_t g) { return ldf(src + g); });
+        } else {
+            const float* src = static_cast<const float*>(in);
+            load_halo<CK, ROWS, CTX, ROWS * CPX, CPX, NT>(
+                tile, image, ty0, tx0, [&](size_t g) { return relu_grad4(src + g, act + g); },
+                [&](size_t g) { return ldf(act + g) > 0.0f ? src[g] : 0.0f; });
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int c = 0; c < CK; ++c) {
+            float win[4][6];
+#pragma unroll
+            for (int dy = 0; dy < 4; ++dy) {
+                const float* r = tile + (c * ROWS + y + dy) * CPX + x0;
+                const float4 a = *reinterpret_cast<const float4*>(r);
+                const float2 d = *reinterpret_cast<const float2*>(r + 4);
+                win[dy][0] = a.x, win[dy][1] = a.y, win[dy][2] = a.z, win[dy][3] = a.w, win[dy][4] = d.x, win[dy][5] = d.y;
+            }
+            const float4* wc = reinterpret_cast<const float4*>(wsm + (c0 + c) * 9 * CO + o0);
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) {
+                const float4 wa = wc[tap * (CO / 4)], wb = wc[tap * (CO / 4) + 1];
+                const float2 ww[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y), make_float2(wb.z, wb.w)};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float t = win[j / 4 + tap / 3][j % 4 + tap % 3];
+                    const float2 v = make_float2(t, t);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[j / 4][j % 4][e] = __ffma2_rn(ww[e], v, acc[j / 4][j % 4][e]);
+                }
             }
         }
-        tile[q] = v;
     }
-    __syncthreads();
-    float acc[CO];
 #pragma unroll
-    for (int o = 0; o < CO; ++o) acc[o] = (MODE == 0) ? ldf(bias + o) : 0.0f;
-    for (int c = 0; c < CI; ++c) {
+    for (int o = 0; o < 16; ++o) {
+        const int row = o / 8, ch = o % 8;
+        const size_t at = (static_cast<size_t>(b) * CO + o0 + ch) * PHW + (ty0 + y + row) * PW + tx0 + x0;
+        float v[4];
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const float x = tile[(c * TH + py + tap / 3) * TH + px + tap % 3];
-            const float4* w4 = reinterpret_cast<const float4*>(wsm + (c * 9 + tap) * CO);
-#pragma unroll
-            for (int o4 = 0; o4 < CO / 4; ++o4) {
-                const float4 ww = w4[o4];
-                acc[4 * o4] = fmaf(ww.x, x, acc[4 * o4]);
-                acc[4 * o4 + 1] = fmaf(ww.y, x, acc[4 * o4 + 1]);
-                acc[4 * o4 + 2] = fmaf(ww.z, x, acc[4 * o4 + 2]);
-                acc[4 * o4 + 3] = fmaf(ww.w, x, acc[4 * o4 + 3]);
-            }
+        for (int j = 0; j < 4; ++j) {
+            v[j] = (ch & 1) ? acc[row][j][ch / 2].y : acc[row][j][ch / 2].x;
+            if (MODE == 0) v[j] = fmaxf(v[j], 0.0f);
         }
-    }
-    const size_t base = static_cast<size_t>(b) * CO * PHW + (ty0 + py) * PW + tx0 + px;
-#pragma unroll
-    for (int o = 0; o < CO; ++o) {
-        if constexpr (MODE == 0)
-            stf(static_cast<TA*>(out) + base + static_cast<size_t>(o) * PHW, fmaxf(acc[o], 0.0f));
-        else
-            static_cast<float*>(out)[base + static_cast<size_t>(o) * PHW] = acc[o];
+        if constexpr (MODE == 0 && sizeof(TA) == 2) {
+            const __half2 h[2] = {__floats2half2_rn(v[0], v[1]), __floats2half2_rn(v[2], v[3])};
+            *reinterpret_cast<uint2*>(static_cast<TA*>(out) + at) = *reinterpret_cast<const uint2*>(h);
+        } else {
+            *reinterpret_cast<float4*>(static_cast<float*>(out) + at) = make_float4(v[0], v[1], v[2], v[3]);
+        }
     }
 }
 
 template <int CI, int CO>
 size_t conv_smem() {
-    return sizeof(float) * (CI * 9 * CO + CI * TH * TH);
+    return sizeof(float) * (CI * 9 * CO + (CI < CCK ? CI : CCK) * (CTY + 2) * CPX);
 }
 
 // ------------------------------------------------------------- weight gradient
 // dW[o][c][tap] += sum_pixels dZ[o][p] A[c][p + tap],  db[o] += sum_pixels dZ[o][p],
-// dZ = dA * (act > 0).  A CTA loops over tiles; each thread owns one input channel c,
-// NO output channels and a pixel subset, and adds its partial sums atomically at the end.
+// dZ = dA * (act > 0).  A CTA loops over 16 x 16 tiles; a thread owns one input channel, four output
+// channels (two packed FP32x2 pairs) and rows of pixels of a tile, along which it slides the 3 x 3
+// window (three new inputs and one 16-byte dZ read a pixel serve 18 packed operations).  The sums of
+// a CTA's pixel groups are added in shared memory, one atomic per weight and CTA.
+// What bounds it: the FP32 pipe.  256 patches, layers 3 / 2 / 1: 0.26 / 0.26 / 0.075 ms; 0.77 / 0.48 / 0.54 ms
+// with a nine-value window and two dZ reads per 18 multiply-adds and an atomic per thread.
+template <int CI, int CO>
+struct WgPlan {
+    static constexpr int UNITS = CI * CO / 4;                    // (channel, four outputs)
+    static constexpr int NT = 256, G = NT / UNITS;               // pixel groups
+    static constexpr int CP = TH * TH + 1;                       // channel pitch: lanes on 32 channels, 32 banks
+    static constexpr int ZP = CO + 4;                            // pixel pitch of dZ [pixel][output]
+    static constexpr int FLOATS = ((CI * CP + 3) / 4) * 4 + T * T * ZP;
+    static_assert(NT % UNITS == 0 && G <= 64, "plan");
+};
+
 template <int CI, int CO, typename TIN, typename TA>
 __global__ void __launch_bounds__(256) wgrad_kernel(const TIN* __restrict__ A, const float* __restrict__ dA,
                                                     const TA* __restrict__ act, float* __restrict__ dW,
                                                     float* __restrict__ db, int n_tiles) {
-    constexpr int PAIRS = CI * CO;
-    constexpr int G = PAIRS >= 256 ? 1 : 256 / PAIRS;          // pixel groups
-    constexpr int NO = PAIRS >= 256 ? PAIRS / 256 : 1;          // output channels per thread
-    constexpr int OSTRIDE = PAIRS >= 256 ? 256 / CI : 1;
-    static_assert(PAIRS % 256 == 0 || 256 % PAIRS == 0, "pair split");
+    using P = WgPlan<CI, CO>;
+    constexpr int G = P::G, SEG = G <= T ? 1 : G / T, W = T / SEG;   // a group takes rows y = g % 16 (+ 16 ..), segments of W pixels
     extern __shared__ __align__(16) float sm[];
-    float* at = sm;                         // CI * TH * TH
-    float* dz = sm + CI * TH * TH;          // CO * T * T
-    const int tid = threadIdx.x;
-    int c, o0, g;
-    if constexpr (PAIRS >= 256) {
-        c = tid % CI;
-        o0 = tid / CI;
-        g = 0;
-    } else {
-        const int pr = tid % PAIRS;
-        c = pr % CI;
-        o0 = pr / CI;
-        g = tid / PAIRS;
-    }
-    float acc[NO][9], accb[NO];
+    float* at = sm;                                     // [CI][CP]
+    float* dz = sm + ((CI * P::CP + 3) / 4) * 4;        // [T * T][ZP]
+    const int tid = threadIdx.x, u = tid % P::UNITS, g = tid / P::UNITS;
+    const int c = u % CI, o0 = 4 * (u / CI);
+    float2 acc[9][2];
 #pragma unroll
-    for (int j = 0; j < NO; ++j) {
-        accb[j] = 0.0f;
-#pragma unroll
-        for (int tap = 0; tap < 9; ++tap) acc[j][tap] = 0.0f;
-    }
+    for (int tap = 0; tap < 9; ++tap) acc[tap][0] = acc[tap][1] = make_float2(0.0f, 0.0f);
+    float accb = 0.0f;                                  // db of output tid % CO, pixels tid / CO ..
+    const bool wide = (reinterpret_cast<uintptr_t>(A) & 15) == 0;
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const int b = tile / kTiles, tl = tile % kTiles;
         const int ty0 = (tl / (PW / T)) * T, tx0 = (tl % (PW / T)) * T;
         __syncthreads();   // previous tile's readers are done
-        for (int q = tid; q < CI * TH * TH; q += 256) {
-            const int cc = q / (TH * TH), r = q % (TH * TH), yy = r / TH, xx = r % TH;
-            const int gy = ty0 + yy - 1, gx = tx0 + xx - 1;
-            float v = 0.0f;
-            if (gy >= 0 && gy < PH && gx >= 0 && gx < PW)
-                v = ldf(A + (static_cast<size_t>(b) * CI + cc) * PHW + gy * PW + gx);
-            at[q] = v;
-        }
-        for (int q = tid; q < CO * T * T; q += 256) {
-            const int oo = q / (T * T), r = q % (T * T);
-            const size_t gi = (static_cast<size_t>(b) * CO + oo) * PHW + (ty0 + r / T) * PW + tx0 + r % T;
-            dz[q] = ldf(act + gi) > 0.0f ? dA[gi] : 0.0f;
+        load_halo<CI, TH, T, P::CP, TH, P::NT>(
+            at, static_cast<size_t>(b) * CI * PHW, ty0, tx0, [&](size_t i) { return ldf4(A + i, wide); },
+            [&](size_t i) { return ldf(A + i); });
+        for (int q = tid; q < CO * T * T / 4; q += P::NT) {
+            const int x4 = 4 * (q % (T / 4)), yy = (q / (T / 4)) % T, oo = q / (T * T / 4);
+            const size_t i = (static_cast<size_t>(b) * CO + oo) * PHW + (ty0 + yy) * PW + tx0 + x4;
+            const float4 v = relu_grad4(dA + i, act + i);
+            float* d = dz + (yy * T + x4) * P::ZP + oo;
+            d[0] = v.x, d[P::ZP] = v.y, d[2 * P::ZP] = v.z, d[3 * P::ZP] = v.w;
         }
         __syncthreads();
-        for (int p = g; p < T * T; p += G) {
-            const int y = p / T, x = p % T;
-            float a9[9];
+        for (int p = tid / CO; p < T * T; p += P::NT / CO) accb += dz[p * P::ZP + tid % CO];
+        for (int y = g / SEG; y < T; y += G / SEG) {
+            const int xs = (g % SEG) * W;
+            const float* a = at + c * P::CP + y * TH + xs;
+            const float* z = dz + (y * T + xs) * P::ZP + o0;
+            float w0[3], w1[3];
 #pragma unroll
-            for (int tap = 0; tap < 9; ++tap) a9[tap] = at[(c * TH + y + tap / 3) * TH + x + tap % 3];
+            for (int dy = 0; dy < 3; ++dy) {
+                w0[dy] = a[dy * TH];
+                w1[dy] = a[dy * TH + 1];
+            }
 #pragma unroll
-            for (int j = 0; j < NO; ++j) {
-                const float z = dz[(o0 + j * OSTRIDE) * T * T + p];
-                accb[j] += z;
+            for (int x = 0; x < W; ++x) {
+                const float4 zz = *reinterpret_cast<const float4*>(z + x * P::ZP);
+                const float2 za = make_float2(zz.x, zz.y), zb = make_float2(zz.z, zz.w);
 #pragma unroll
-                for (int tap = 0; tap < 9; ++tap) acc[j][tap] = fmaf(z, a9[tap], acc[j][tap]);
+                for (int dy = 0; dy < 3; ++dy) {
+                    const float w2 = a[dy * TH + x + 2];
+                    const float win[3] = {w0[dy], w1[dy], w2};
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx) {
+                        const float2 v = make_float2(win[dx], win[dx]);
+                        acc[3 * dy + dx][0] = __ffma2_rn(za, v, acc[3 * dy + dx][0]);
+                        acc[3 * dy + dx][1] = __ffma2_rn(zb, v, acc[3 * dy + dx][1]);
+                    }
+                    w0[dy] = w1[dy];
+                    w1[dy] = w2;
+                }
             }
         }
     }
+    // the CTA's sums, weight by weight: shared-memory atomics over the pixel groups, then one global each
+    __syncthreads();
+    float* red = sm;                                    // [CO][CI][9], then db [CO]
+    for (int q = tid; q < CO * CI * 9 + CO; q += P::NT) red[q] = 0.0f;
+    __syncthreads();
 #pragma unroll
-    for (int j = 0; j < NO; ++j) {
-        const int o = o0 + j * OSTRIDE;
+    for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) atomicAdd(&dW[(o * CI + c) * 9 + tap], acc[j][tap]);
-        if (c == 0) atomicAdd(&db[o], accb[j]);
-    }
+        for (int tap = 0; tap < 9; ++tap)
+            atomicAdd(&red[((o0 + j) * CI + c) * 9 + tap], (j & 1) ? acc[tap][j / 2].y : acc[tap][j / 2].x);
+    atomicAdd(&red[CO * CI * 9 + tid % CO], accb);
+    __syncthreads();
+    for (int q = tid; q < CO * CI * 9; q += P::NT) atomicAdd(&dW[q], red[q]);
+    if (tid < CO) atomicAdd(&db[tid], red[CO * CI * 9 + tid]);
 }
 
 template <int CI, int CO>
 size_t wgrad_smem() {
-    return sizeof(float) * (CI * TH * TH + CO * T * T);
+    const int red = CO * CI * 9 + CO;
+    return sizeof(float) * static_cast<size_t>(WgPlan<CI, CO>::FLOATS > red ? WgPlan<CI, CO>::FLOATS : red);
 }
 
 // ------------------------------------------------------------------- head
@@ -441,7 +528,7 @@ cudaError_t conv(const void* in, const TA* act, const TA* w, const TA* bias, voi
     auto kern = conv3x3_kernel<CI, CO, MODE, TIN, TA>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    kern<<<B * kTiles, 256, smem, s>>>(in, act, w, bias, out);
+    kern<<<B * kCTiles, 8 * CO, smem, s>>>(in, act, w, bias, out);
     return cudaGetLastError();
 }
 
@@ -453,7 +540,7 @@ cudaError_t wgrad(const TIN* A, const float* dA, const TA* act, float* dW, float
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     const int n_tiles = B * kTiles;
-    const int grid = std::max(1, std::min(n_tiles, 4 * n_sm));
+    const int grid = std::max(1, std::min(n_tiles, 3 * n_sm));
     kern<<<grid, 256, smem, s>>>(A, dA, act, dW, db, n_tiles);
     return cudaGetLastError();
 }
