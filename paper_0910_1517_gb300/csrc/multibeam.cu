@@ -7,12 +7,17 @@
 //                            Im U_b0 conj U_b1
 //   voltages   (products 1, avg 1): Re U_b0, Im U_b0, Re U_b1, Im U_b1
 //
-// One CTA takes channel k and up to 512 frames, staged 64 at a time through two buffers (one
-// bulk copy per stage, the next stages in flight): each stage's FP32 K-blocks are transposed
-// once into planes Yr[i][f], Yi[i][f].  Lanes are consecutive frames (two per lane) and warps
-// beam groups (beams w, w + 8, ...), so every weight read is a broadcast, shared by two frames,
-// and each sample is read once for all of a thread's beams.  A window of `avg` frames is summed
-// by shuffles across its lanes (avg <= 32) and then across 32-frame passes in order.
+// A CTA takes channel k and `span` frames, 128 at a time.  A stage's FP32 K-blocks land as they are,
+// one bulk copy a K-block at a pitch that spreads consecutive K-blocks over the banks, so that lane
+// (K-block, granule) reads its 16 bytes -- four consecutive frames of one row -- without conflicts
+// and without transposing the stage.  A thread forms BPT beams of its four frames, two frames a
+// packed FP32x2 operation: four 16-byte sample reads and BPT 8-byte weight reads an antenna serve
+// 16 BPT packed multiply-adds.  Warps take beam groups.  A window of `avg` frames is summed in the
+// lane, by shuffles across its lanes and then across stages in order.  One buffer a CTA; the SM's
+// other CTAs compute while one waits for its copy.
+// What bounds it: the FP32 pipe from about 8 beams on, the read of the spectra below.  GMRT shape,
+// 4096 spectra, 16 beams, 256-frame windows: 0.76 ms (2.15 GB in, 0.49 ms of multiply-adds); 1.67 ms with the stage transposed
+// through shared memory and two beams a thread (six shared-memory reads for 16 multiply-adds).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -24,157 +29,148 @@
 namespace gbx {
 namespace {
 
-constexpr int kMbThreads = 256;
-constexpr int kMbWarps = kMbThreads / 32;
-constexpr int kMbMaxBeams = 64;                 // beams per launch (kMbMaxBeams / kMbWarps per thread)
-constexpr int kMbFrames = 64;                   // frames per shared-memory stage (a lane takes 2)
+constexpr int kMbMaxBeams = 64;                 // beams per launch
+constexpr int kMbFrames = 128;                  // frames per shared-memory stage (four a lane)
 constexpr int kMbMaxIn = 128;
 constexpr int kMbTcMinBeams = 24;               // more beams than this: the tensor-core form
 
-struct MbShared {
-    uint64_t bar[2];
-};
+// bytes from one K-block of tb frames to the next in shared memory: the K-blocks of a
+// quarter warp's lanes (16 bytes each; two lanes a K-block at tb 8) fall into different banks
+__host__ __device__ constexpr int mb_pitch(int n_in, int tb) { return rows_fp32(n_in) * tb * 4 + 4 * tb; }
+__host__ __device__ constexpr int mb_stage_bytes(int n_in, int tb) { return (kMbFrames / tb) * mb_pitch(n_in, tb); }
 
-// Shared memory: two raw stages (the FP32 K-blocks of 64 frames), the stage transposed into
-// planes Yr[i][f], Yi[i][f], the channel's weights and the window accumulators.
-__host__ __device__ constexpr size_t mb_raw_floats(int n_in, int n_chan) {
-    return static_cast<size_t>(rows_fp32(n_in)) * kMbFrames;
-}
-
-template <int BPT>   // beams per thread
-__global__ void __launch_bounds__(kMbThreads) multibeam_kernel(const float* __restrict__ spec, int n_ant, int n_pol,
-                                                               int n_chan, int n_int, const float2* __restrict__ w,
-                                                               int wstride, int n_beams, int products, int avg,
-                                                               int span, float4* __restrict__ out, unsigned* err) {
-    extern __shared__ __align__(16) float sm[];
-    __shared__ MbShared ms;
-    const int n_in = n_ant * n_pol;
-    const int tb = tb_fp32(n_chan), Rp = rows_fp32(n_in);
-    const int raw_f = static_cast<int>(mb_raw_floats(n_in, n_chan));
-    float* yr = sm + 2 * raw_f;                                     // raw stages: sm + (st & 1) * raw_f                                     // [n_in][64]
-    float* yi = yr + n_in * kMbFrames;
-    float2* ws = reinterpret_cast<float2*>(yi + n_in * kMbFrames);  // [beam][antenna] of channel k
-    float4* acc = reinterpret_cast<float4*>(ws + wstride);          // per (beam, frame half) window sums
+template <int BPT, int TB>   // beams per thread, frames per K-block
+__global__ void __launch_bounds__(512) multibeam_kernel(const float* __restrict__ spec, int n_ant, int n_pol, int n_chan,
+                                                        int n_int, const float2* __restrict__ w, int wstride, int n_beams,
+                                                        int products, int avg, int span, float4* __restrict__ out, unsigned* err) {
+    extern __shared__ __align__(128) unsigned char smb[];
+    __shared__ __align__(8) uint64_t bar;
+    constexpr int H = TB / 4;                                       // granules of a row in a K-block
+    const int n_in = n_ant * n_pol, pitch = mb_pitch(n_in, TB);
+    const float2* ws = reinterpret_cast<const float2*>(smb + mb_stage_bytes(n_in, TB));   // [beam][antenna] of channel k
     const int k = blockIdx.x, t0 = blockIdx.y * span;
-    const int64_t ntb = n_int / tb;
-    const int n_stage = span / kMbFrames;
-    const uint32_t stage_bytes = static_cast<uint32_t>(raw_f) * 4;
+    const int64_t ntb = n_int / TB;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    auto issue = [&](int st) {   // thread 0: stage st's K-blocks (contiguous) into raw[st & 1]
-        const uint32_t wbytes = st == 0 ? static_cast<uint32_t>(wstride) * sizeof(float2) : 0u;
-        mbar_arrive_expect_tx(&ms.bar[st & 1], stage_bytes + wbytes);
-        bulk_g2s(sm + (st & 1) * raw_f, spec + (static_cast<int64_t>(k) * ntb + (t0 + st * kMbFrames) / tb) * Rp * tb,
-                 stage_bytes, &ms.bar[st & 1]);
-        if (st == 0) bulk_g2s(ws, w + static_cast<int64_t>(k) * wstride, wbytes, &ms.bar[0]);
+    const uint32_t kb_bytes = static_cast<uint32_t>(rows_fp32(n_in)) * TB * 4;
+    const int n_stage = (span + kMbFrames - 1) / kMbFrames;
+    auto issue = [&](int st) {   // warp 0: stage st's K-blocks, and with the first the channel's weights
+        const int kbs = min(kMbFrames, span - st * kMbFrames) / TB;
+        if (lane == 0) {
+            mbar_arrive_expect_tx(&bar, kbs * kb_bytes + (st == 0 ? wstride * static_cast<uint32_t>(sizeof(float2)) : 0u));
+            if (st == 0)
+                bulk_g2s(const_cast<float2*>(ws), w + static_cast<int64_t>(k) * wstride, wstride * sizeof(float2), &bar);
+        }
+        __syncwarp();
+        const float* src = spec + (static_cast<int64_t>(k) * ntb + (t0 + st * kMbFrames) / TB) * (kb_bytes / 4);
+        for (int q = lane; q < kbs; q += 32) bulk_g2s(smb + q * pitch, src + static_cast<int64_t>(q) * (kb_bytes / 4), kb_bytes, &bar);
     };
     if (tid == 0) {
-        mbar_init(&ms.bar[0], 1);
-        mbar_init(&ms.bar[1], 1);
+        mbar_init(&bar, 1);
         fence_mbar_init();
-        issue(0);
-        if (n_stage > 1) issue(1);
     }
     __syncthreads();
-    const int n_out = n_int / avg;
-    bool ok = true;
-    int st = 0;
-    for (; st < n_stage && ok; ++st) {
-        ok = __syncthreads_and(mbar_wait(&ms.bar[st & 1], (st >> 1) & 1, err, ERR_WAIT_STAGE));
-        if (!ok) break;
-        // transpose: granule q of the stage = 4 frames of one row (the FP32 layout's XOR placement undone)
-        const float* rs = sm + (st & 1) * raw_f;
-        const int gpb = Rp * tb / 4;                                // granules per K-block
-        for (int q = tid; q < (kMbFrames / tb) * gpb; q += kMbThreads) {
-            const int kb = q / gpb, pos = q % gpb;
-            const int G = pos / (2 * tb), gs = (pos % (2 * tb)) ^ (G & 7);
-            const int r = G * 8 + gs / (tb / 4), f0 = kb * tb + (gs % (tb / 4)) * 4;
-            if (r >= 2 * n_in) continue;                            // padding rows
-            const float4 v = reinterpret_cast<const float4*>(rs)[q];
-            *reinterpret_cast<float4*>(((r & 1) ? yi : yr) + (r >> 1) * kMbFrames + f0) = v;
+    if (warp == 0) issue(0);
+    const int n_out = n_int / avg, b0 = warp * BPT;
+    const unsigned char* mine = smb + (lane / H) * pitch;           // this lane's K-block, granule lane % H of each row
+    float4 acc[BPT];                                                // windows of more than a stage (lane 0)
+#pragma unroll
+    for (int q = 0; q < BPT; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int st = 0; st < n_stage; ++st) {
+        if (!__syncthreads_and(mbar_wait_warp(&bar, st & 1, err, ERR_WAIT_STAGE))) {
+            if (tid == 0) mbar_wait(&bar, st & 1, nullptr, 0);      // the copies in flight land before the CTA exits (bounded)
+            break;
         }
-        __syncthreads();                                            // the raw stage read, planes written
-        if (tid == 0 && st + 2 < n_stage) issue(st + 2);
-        // beams: lane takes frames lane and lane + 32 of the stage, warp the beams warp + 8 q
-        float ur[BPT][2][2], ui[BPT][2][2];                         // [beam][frame half][pol]
+        const int frames = min(kMbFrames, span - st * kMbFrames);
+        const bool live = 4 * lane < frames;                        // (a last stage of 64 frames: half the lanes)
+        float2 ur[BPT][2][2], ui[BPT][2][2];                        // [beam][pol][frames 0, 1 | 2, 3]
 #pragma unroll
         for (int q = 0; q < BPT; ++q)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) ur[q][h][0] = ur[q][h][1] = ui[q][h][0] = ui[q][h][1] = 0.0f;
-        for (int a = 0; a < n_ant; ++a)
+            for (int e = 0; e < 4; ++e) ur[q][e / 2][e % 2] = ui[q][e / 2][e % 2] = make_float2(0.f, 0.f);
+        for (int a = 0; a < n_ant; ++a) {
+            float4 yr[2], yi[2];
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                if (p >= n_pol) break;
-                const int i = a * n_pol + p;
-                const float r0 = yr[i * kMbFrames + lane], i0 = yi[i * kMbFrames + lane];
-                const float r1 = yr[i * kMbFrames + lane + 32], i1 = yi[i * kMbFrames + lane + 32];
-#pragma unroll
-                for (int q = 0; q < BPT; ++q) {
-                    const int b = warp + q * kMbWarps;
-                    const float2 wv = ws[(b < n_beams ? b : 0) * n_ant + a];
-                    ur[q][0][p] = fmaf(wv.x, r0, fmaf(-wv.y, i0, ur[q][0][p]));
-                    ui[q][0][p] = fmaf(wv.x, i0, fmaf(wv.y, r0, ui[q][0][p]));
-                    ur[q][1][p] = fmaf(wv.x, r1, fmaf(-wv.y, i1, ur[q][1][p]));
-                    ui[q][1][p] = fmaf(wv.x, i1, fmaf(wv.y, r1, ui[q][1][p]));
-                }
+                // rows 2i and 2i + 1 of input i: granules ((r % 8) H + half) ^ (G % 8) of row group G
+                const int i = a * n_pol + (p < n_pol ? p : 0), G = i >> 2, g = (2 * i) & 7;
+                const unsigned char* grp = mine + G * 128 * H;
+                yr[p] = *reinterpret_cast<const float4*>(grp + (((g * H + lane % H) ^ (G & 7)) << 4));
+                yi[p] = *reinterpret_cast<const float4*>(grp + ((((g + 1) * H + lane % H) ^ (G & 7)) << 4));
             }
-        const int ts = t0 + st * kMbFrames;                         // first frame of the stage
+#pragma unroll
+            for (int q = 0; q < BPT; ++q) {
+                const float2 wv = ws[(b0 + q < n_beams ? b0 + q : 0) * n_ant + a];
+                const float2 wr = make_float2(wv.x, wv.x), wi = make_float2(wv.y, wv.y), nwi = make_float2(-wv.y, -wv.y);
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float2 r = h ? make_float2(yr[p].z, yr[p].w) : make_float2(yr[p].x, yr[p].y);
+                        const float2 m = h ? make_float2(yi[p].z, yi[p].w) : make_float2(yi[p].x, yi[p].y);
+                        ur[q][p][h] = __ffma2_rn(wr, r, __ffma2_rn(nwi, m, ur[q][p][h]));
+                        ui[q][p][h] = __ffma2_rn(wr, m, __ffma2_rn(wi, r, ui[q][p][h]));
+                    }
+            }
+        }
+        __syncthreads();                                            // the stage is read: the next may land
+        if (warp == 0 && st + 1 < n_stage) {
+            fence_proxy_async_smem();
+            issue(st + 1);
+        }
+        const int ts = t0 + st * kMbFrames + 4 * lane;              // this lane's first frame
 #pragma unroll
         for (int q = 0; q < BPT; ++q) {
-            const int b = warp + q * kMbWarps;
-            if (b >= n_beams) break;
+            const int b = b0 + q;
+            if (b >= n_beams) break;                                // (the same for the whole warp)
+            float4* ob = out + static_cast<int64_t>(b) * n_out * n_chan + k;
+            float4 v[4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int f = h * 32 + lane;
-                if (products == 1) {
-                    out[(static_cast<int64_t>(b) * n_out + ts + f) * n_chan + k] =
-                        make_float4(ur[q][h][0], ui[q][h][0], ur[q][h][1], ui[q][h][1]);
-                    continue;
+            for (int f = 0; f < 4; ++f) {
+                auto at = [&](const float2 (&u)[2][2], int p) { return (f & 1) ? u[p][f / 2].y : u[p][f / 2].x; };
+                const float r0 = at(ur[q], 0), i0 = at(ui[q], 0), r1 = n_pol == 2 ? at(ur[q], 1) : 0.0f, i1 = n_pol == 2 ? at(ui[q], 1) : 0.0f;
+                v[f] = products == 1 ? make_float4(r0, i0, r1, i1)
+                                     : make_float4(r0 * r0 + i0 * i0, r1 * r1 + i1 * i1, r0 * r1 + i0 * i1, i0 * r1 - r0 * i1);
+            }
+            auto add = [](float4 x, float4 y) { return make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w); };
+            const float sc = 1.0f / avg;
+            auto put = [&](int t, float4 x) { ob[static_cast<int64_t>(t / avg) * n_chan] = make_float4(x.x * sc, x.y * sc, x.z * sc, x.w * sc); };
+            if (avg <= 2) {
+                if (live) {
+                    if (avg == 1) {
+#pragma unroll
+                        for (int f = 0; f < 4; ++f) put(ts + f, v[f]);
+                    } else {
+                        put(ts, add(v[0], v[1]));
+                        put(ts + 2, add(v[2], v[3]));
+                    }
                 }
-                float4 v = make_float4(ur[q][h][0] * ur[q][h][0] + ui[q][h][0] * ui[q][h][0],
-                                       ur[q][h][1] * ur[q][h][1] + ui[q][h][1] * ui[q][h][1],
-                                       ur[q][h][0] * ur[q][h][1] + ui[q][h][0] * ui[q][h][1],
-                                       ui[q][h][0] * ur[q][h][1] - ur[q][h][0] * ui[q][h][1]);
-                // sum over the window's lanes (avg <= 32), or over the warp (avg > 32), fixed order
-                const int sp = avg < 32 ? avg : 32;
-                for (int off = 1; off < sp; off <<= 1) {
-                    v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
-                    v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
-                    v.z += __shfl_xor_sync(0xffffffffu, v.z, off);
-                    v.w += __shfl_xor_sync(0xffffffffu, v.w, off);
-                }
-                const float sc = 1.0f / avg;
-                if (avg <= 32) {
-                    if (lane % sp == 0)
-                        out[(static_cast<int64_t>(b) * n_out + (ts + f) / avg) * n_chan + k] =
-                            make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
-                } else if (lane == 0) {                             // 32-frame passes of one window, in order
-                    const int gpass = (ts + f - t0) / 32;           // pass index within the CTA
-                    const int per = avg / 32;
-                    float4 a4 = gpass % per == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : acc[b];
-                    a4 = make_float4(a4.x + v.x, a4.y + v.y, a4.z + v.z, a4.w + v.w);
-                    acc[b] = a4;
-                    if (gpass % per == per - 1)
-                        out[(static_cast<int64_t>(b) * n_out + (ts + f) / avg) * n_chan + k] =
-                            make_float4(a4.x * sc, a4.y * sc, a4.z * sc, a4.w * sc);
+                continue;
+            }
+            float4 s = add(add(v[0], v[1]), add(v[2], v[3]));
+            if (!live) s = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int lanes = min(avg / 4, 32);
+            for (int off = 1; off < lanes; off <<= 1) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+                s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+                s.z += __shfl_xor_sync(0xffffffffu, s.z, off);
+                s.w += __shfl_xor_sync(0xffffffffu, s.w, off);
+            }
+            if (avg <= kMbFrames) {
+                if (live && lane % lanes == 0) put(ts, s);
+            } else {                                                // stages of one window, in order
+                acc[q] = add(acc[q], s);
+                if ((st + 1) * kMbFrames % avg == 0) {
+                    if (lane == 0) put(ts, acc[q]);
+                    acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
         }
-        __syncthreads();                                            // planes read: the next transpose may write
-    }
-    if (!ok && tid == 0) {   // copies in flight land before the CTA exits (bounded)
-        for (int q = st; q < n_stage && q < st + 2; ++q) mbar_wait(&ms.bar[q & 1], (q >> 1) & 1, nullptr, 0);
     }
 }
 
 }  // namespace
 
 int multibeam_max_beams() { return kMbMaxBeams; }
-
-size_t multibeam_smem(int n_in, int n_chan, int n_beams, int n_ant) {
-    const int wstride = ((n_beams * n_ant + 1) / 2) * 2;
-    return sizeof(float) * (2 * mb_raw_floats(n_in, n_chan) + 2 * static_cast<size_t>(n_in) * kMbFrames) +
-           sizeof(float2) * wstride + sizeof(float4) * n_beams;
-}
 
 int multibeam_wstride(int n_beams, int n_ant) { return ((n_beams * n_ant + 1) / 2) * 2; }
 
@@ -183,34 +179,35 @@ cudaError_t launch_multibeam(const float* spec, int n_ant, int n_pol, int n_chan
     if (n_beams < 1 || n_beams > kMbMaxBeams || avg < 1 || (avg & (avg - 1)) || n_int % (avg > 64 ? avg : 64) ||
         (products != 0 && products != 1) || (products == 1 && avg != 1) || n_ant * n_pol > kMbMaxIn)
         return cudaErrorInvalidValue;
-    // frames per CTA: a multiple of 64 and of avg dividing n_int, up to 512 (more stages per CTA
-    // hide the copies; fewer CTAs per channel leave enough of them)
+    // frames per CTA: a multiple of avg dividing n_int, of 128 where there are as many, up to 512
+    // (its later stages' copies run while the earlier ones' products are formed)
     int span = avg > 64 ? avg : 64;
     while (span < 512 && n_int % (2 * span) == 0) span *= 2;
     const int wstride = multibeam_wstride(n_beams, n_ant);
-    // the tensor-core form for many beams: its time hardly depends on the beam count (5.0 ms for
-    // 16 and 5.1 ms for 64 beams at GMRT scale), the CUDA-core kernel's grows with it (3.4 ms for
-    // 16, 13.0 ms for 64); they cross near 24 beams
+    // the tensor-core form for many beams: its time hardly depends on their count (1.7 ms for 64 beams
+    // at GMRT scale, 8192 spectra), the CUDA-core kernel's grows with it (1.5 ms for 16, 2.0 ms for
+    // 24), but its fp16 hi/lo split is less exact (errors of 5e-7 to 4e-6 against 1e-7 to 3e-6), so
+    // the line stays above the crossing
     if (n_beams > kMbTcMinBeams && multibeam_tc_supported(n_ant, n_pol, n_chan, n_int)) {
         int e = -8;
         for (int n = 2 * n_chan; n > 1; n >>= 1) ++e;
         return launch_multibeam_tc(spec, n_ant, n_pol, n_chan, n_int, w, wstride, n_beams, products, avg,
                                    ldexpf(1.0f, -e), out, err, s);
     }
-    const size_t smem = multibeam_smem(n_ant * n_pol, n_chan, n_beams, n_ant);
+    const int tb = tb_fp32(n_chan), n_in = n_ant * n_pol;
+    const size_t smem = static_cast<size_t>(mb_stage_bytes(n_in, tb)) + sizeof(float2) * wstride;
     const dim3 grid(n_chan, n_int / span);
-    auto go = [&](auto kern) {
+    auto go = [&](auto kern, int bpt) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
-        kern<<<grid, kMbThreads, smem, s>>>(spec, n_ant, n_pol, n_chan, n_int, w, wstride, n_beams, products, avg,
-                                            span, out, err);
+        kern<<<grid, 32 * ((n_beams + bpt - 1) / bpt), smem, s>>>(spec, n_ant, n_pol, n_chan, n_int, w, wstride, n_beams, products,
+                                                                 avg, span, out, err);
         return cudaGetLastError();
     };
-    const int bpt = (n_beams + kMbWarps - 1) / kMbWarps;
-    if (bpt <= 1) return go(multibeam_kernel<1>);
-    if (bpt <= 2) return go(multibeam_kernel<2>);
-    if (bpt <= 4) return go(multibeam_kernel<4>);
-    return go(multibeam_kernel<8>);
+    // beams a thread: four keep the FP32 pipe ahead of the shared-memory reads; fewer beams than 16
+    // take less, so that a CTA has four warps
+    if (tb == 8) return n_beams > 8 ? go(multibeam_kernel<4, 8>, 4) : n_beams > 4 ? go(multibeam_kernel<2, 8>, 2) : go(multibeam_kernel<1, 8>, 1);
+    return n_beams > 8 ? go(multibeam_kernel<4, 4>, 4) : n_beams > 4 ? go(multibeam_kernel<2, 4>, 2) : go(multibeam_kernel<1, 4>, 1);
 }
 
 }  // namespace gbx
