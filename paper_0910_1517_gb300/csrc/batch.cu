@@ -38,6 +38,7 @@ struct corr_batch {
     int64_t* d_g0 = nullptr;
     FeParams fe_p[kMaxSub] = {};              // F-engine parameters of the next replay
     FeParams cap_p[kMaxSub] = {};             // ... and those the graph was captured with
+    int cap_dump[kMaxSub] = {};
     cudaGraphNode_t fe_node[kMaxSub] = {};    // the F-engine kernel node of each branch
     cudaKernelNodeParams fe_kp[kMaxSub] = {};
     XtBatch* h_xt = nullptr;     // pinned, one one-entry table per sub-array
@@ -101,7 +102,8 @@ FeParams fe_params(corr* h, const int8_t* x, int64_t ld, int64_t n_avail) {
     fp.ff = h->d_ff;
     fp.wcoh = h->d_wcoh;
     fp.ginc = h->d_ginc;
-    fp.scale = h->d_scale;
+    if (tc_mode(h->xmode)) fp.scale = h->d_scale;
+    else fp.dump = h->d_dump_part;
     fp.spec = h->d_spec;
     fp.beams = h->d_beams_raw;
     fp.tw = h->d_tw;
@@ -145,8 +147,7 @@ bool capture_branch(corr_batch* b, int q, cudaStream_t s) {
         ok = launch_xengine_fp32(xp, b->n_sm, s) == cudaSuccess;
     }
     if (ok && h->dump > 0 && b->xmode == CORR_FP32)
-        ok = launch_power_dumps(static_cast<const float*>(h->d_spec), h->n_in, h->n_chan, h->n_int, h->dump,
-                                h->d_power, s) == cudaSuccess;
+        ok = launch_power_dumps(h->d_dump_part, h->n_in, h->n_chan, h->n_int, h->dump, h->d_power, s) == cudaSuccess;
     if (ok && h->beam_avg > 1)
         ok = launch_beam_average(h->d_beams_raw, h->d_beams, h->n_int, h->n_chan, h->beam_avg, s) == cudaSuccess;
     return ok;
@@ -184,7 +185,10 @@ int capture(corr_batch* b) {
     }
     b->graph = g;
     BCU(cudaGraphInstantiate(&b->exec, g, 0));
-    for (int q = 0; q < b->n_sub; ++q) b->cap_p[q] = b->fe_p[q];
+    for (int q = 0; q < b->n_sub; ++q) {
+        b->cap_p[q] = b->fe_p[q];
+        b->cap_dump[q] = b->h[q]->dump;
+    }
     for (int q = 0; q < b->n_sub; ++q) BCU(cudaGraphKernelNodeGetParams(b->fe_node[q], &b->fe_kp[q]));
     return CORR_OK;
 }
@@ -302,6 +306,8 @@ int corr_batch_integrate_device(corr_batch_t* b, const int8_t* const* x, const i
     for (int q = 0; q < b->n_sub; ++q)
         if (fengine_clustered(b->h[q]->n_chan, b->fmode[q]) && std::memcmp(&b->fe_p[q], &b->cap_p[q], sizeof(FeParams)))
             recapture = true;
+    for (int q = 0; q < b->n_sub; ++q)   // the dumps' buffers are the capture's
+        if (b->fe_p[q].dump != b->cap_p[q].dump || b->h[q]->dump != b->cap_dump[q]) recapture = true;
     if (recapture)
         if (int rc = capture(b)) return rc;
     for (int q = 0; q < b->n_sub; ++q) {   // this integration's sample pointers into the F-engine nodes

@@ -175,7 +175,8 @@ int gbx::run_integration(corr* h, const int8_t* x, int64_t ld, int64_t n_avail, 
     fp.ff = h->d_ff;
     fp.wcoh = h->d_wcoh;
     fp.ginc = h->d_ginc;
-    fp.scale = h->d_scale;
+    if (h->xmode == CORR_I8 || h->xmode == CORR_F16) fp.scale = h->d_scale;
+    else fp.dump = h->d_dump_part;
     fp.spec = h->d_spec;
     fp.beams = h->d_beams_raw;
     fp.tw = h->d_tw;
@@ -222,8 +223,7 @@ int gbx::run_integration(corr* h, const int8_t* x, int64_t ld, int64_t n_avail, 
         CU(launch_xengine_tc_table(h->out_buf == 1 ? h->xtab_b1 : h->d_xtab, h->n_items, h->n_sm, s,
                                    h->xmode == CORR_FP32TC ? xt_form_f32(h->n_in) : fmode == OUT_I8B ? XT_FORM_I8 : XT_FORM_F16));
     if (h->dump > 0) {
-        CU(launch_power_dumps(static_cast<const float*>(h->d_spec), h->n_in, h->n_chan, h->n_int, h->dump,
-                              h->d_power, s, fmode == OUT_F32Q));
+        CU(launch_power_dumps(h->d_dump_part, h->n_in, h->n_chan, h->n_int, h->dump, h->d_power, s));
     }
     if (int rc = mark(h, 3, s)) return rc;
     if (h->beam_avg > 1) CU(launch_beam_average(h->d_beams_raw, h->d_beams, h->n_int, h->n_chan, h->beam_avg, s));
@@ -530,6 +530,7 @@ int corr_destroy(corr_t* h) {
     if (h->cstream) cudaStreamSynchronize(h->cstream);
     if (h->ustream) cudaStreamSynchronize(h->ustream);
     if (h->ostream) cudaStreamSynchronize(h->ostream);
+    if (h->d_dump_part && h->d_dump_part != h->d_power) cudaFree(h->d_dump_part);
     if (h->d_power) cudaFree(h->d_power);
     if (h->d_noise) cudaFree(h->d_noise);
     if (h->d_blank) cudaFree(h->d_blank);
@@ -982,12 +983,17 @@ int corr_set_power_dump(corr_t* h, int dump) {
     if (dump < 0 || (dump > 0 && (dump % tb_fp32(h->n_chan) || h->n_int % dump)))
         return fail(CORR_E_INVAL, "dump must be 0 or a multiple of %d dividing n_int", tb_fp32(h->n_chan));
     CU(cudaStreamSynchronize(h->stream));
+    if (h->d_dump_part && h->d_dump_part != h->d_power) cudaFree(h->d_dump_part);
     if (h->d_power) cudaFree(h->d_power);
-    h->d_power = nullptr;
-    h->dump = dump;
+    h->d_power = h->d_dump_part = nullptr;
+    h->dump = 0;
     if (dump > 0) {
         CU(dalloc(&h->d_power, static_cast<size_t>(h->n_in) * (h->n_int / dump) * h->n_chan));
         CU(cudaMemset(h->d_power, 0, sizeof(float) * h->n_in * (h->n_int / dump) * h->n_chan));
+        const int tb = tb_fp32(h->n_chan);
+        if (dump == tb) h->d_dump_part = h->d_power;
+        else CU(dalloc(&h->d_dump_part, static_cast<size_t>(h->n_in) * (h->n_int / tb) * h->n_chan));
+        h->dump = dump;
     }
     return CORR_OK;
 }

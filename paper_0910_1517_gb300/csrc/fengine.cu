@@ -40,35 +40,20 @@ __global__ void twiddle_kernel(int n_fft, int count, float2* __restrict__ tw) {
     }
 }
 
-// grid.x: dumps, grid.y: 32-channel groups; lane = channel, warp rows step over inputs
-__global__ void power_dump_kernel(const float* __restrict__ spec, int n_in, int n_chan, int n_int, int dump,
-                                  float* __restrict__ P, bool quad) {
-    const int d = blockIdx.x, k = blockIdx.y * 32 + threadIdx.x;
-    if (k >= n_chan) return;
-    const int tb = tb_fp32(n_chan);
-    const int Rp = rows_fp32(n_in), ntb = n_int / tb, n_dump = n_int / dump;
-    const int kb0 = d * dump / tb, nkb = dump / tb;
-    for (int i = threadIdx.y; i < n_in; i += blockDim.y) {
-        float acc = 0.0f;
-        for (int kb = kb0; kb < kb0 + nkb; ++kb) {
-            if (quad) {   // one 64-byte piece: 8 re then 8 im values, summed in the order of the other layout
-                const float4* pc = reinterpret_cast<const float4*>(spec + f32q_piece(k, kb, i, ntb, n_in));
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const float4 v = pc[(m >> 1) + 2 * (m & 1)];   // re 0-3, im 0-3, re 4-7, im 4-7
-                    acc += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-                }
-                continue;
-            }
-            const float* blk = spec + (static_cast<int64_t>(k) * ntb + kb) * Rp * tb;
-            for (int e = 0; e < tb; e += 4) {            // one 4-frame granule of each row at a time
-                const float4 re = *reinterpret_cast<const float4*>(blk + fp32_off(2 * i, e, tb));
-                const float4 im = *reinterpret_cast<const float4*>(blk + fp32_off(2 * i + 1, e, tb));
-                acc += re.x * re.x + re.y * re.y + re.z * re.z + re.w * re.w;
-                acc += im.x * im.x + im.y * im.y + im.z * im.z + im.w * im.w;
-            }
+// Four channels a thread; n sums a dump.  What bounds it: reading the sums, a sixteenth of the
+// spectra.  GMRT shape, 60 inputs, 4096 spectra: the whole integration 0.42 ms shorter than with a
+// kernel that summed the 2 GB of spectra themselves (0.49 ms).
+__global__ void power_dump_kernel(const float4* __restrict__ part, int n, int64_t n_out, int n_quad, float4* __restrict__ P) {
+    for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < n_out;
+         q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const float4* src = part + q / n_quad * n * n_quad + q % n_quad;   // dump q / n_quad of all inputs' in order
+        float4 a = src[0];
+#pragma unroll 4
+        for (int j = 1; j < n; ++j) {
+            const float4 v = src[static_cast<int64_t>(j) * n_quad];
+            a.x += v.x, a.y += v.y, a.z += v.z, a.w += v.w;
         }
-        P[(static_cast<int64_t>(i) * n_dump + d) * n_chan + k] = acc;
+        P[q] = a;
     }
 }
 
@@ -121,12 +106,13 @@ cudaError_t launch_phasor_setup(int n_ant, int n_chan, int n_fft, int n_int, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_power_dumps(const float* spec, int n_in, int n_chan, int n_int, int dump, float* P,
-                               cudaStream_t s, bool quad) {
-    const int tb = tb_fp32(n_chan);
+cudaError_t launch_power_dumps(const float* part, int n_in, int n_chan, int n_int, int dump, float* P, cudaStream_t s) {
+    const int tb = tb_fp32(n_chan), n = dump / tb, n_quad = n_chan / 4;
     if (dump < tb || dump % tb || n_int % dump) return cudaErrorInvalidValue;
-    const dim3 grid(n_int / dump, (n_chan + 31) / 32), block(32, 8);
-    power_dump_kernel<<<grid, block, 0, s>>>(spec, n_in, n_chan, n_int, dump, P, quad);
+    if (n == 1) return cudaSuccess;
+    const int64_t n_out = static_cast<int64_t>(n_in) * (n_int / dump) * n_quad;
+    const int grid = static_cast<int>(std::min<int64_t>((n_out + 255) / 256, 8192));
+    power_dump_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float4*>(part), n, n_out, n_quad, reinterpret_cast<float4*>(P));
     return cudaGetLastError();
 }
 

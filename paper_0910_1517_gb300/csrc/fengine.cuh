@@ -64,7 +64,11 @@ struct FeParams {
     const float2* ff;      // [n_ant][n_int] fringe phasor exp(-i phi_a(g0 + t))
     const float2* wcoh;    // [n_ant][n_chan] coherent-beam weight g_a exp(i theta_ak), 0 if unselected
     const float* ginc;     // [n_ant] incoherent weight g_a^2, 0 if unselected
-    const float* scale;    // [n_in][n_chan] requantisation scales (I8 / F16)
+    union {                // (a field of its own for the dumps made every kernel here spill)
+        const float* scale;   // I8 / F16: [n_in][n_chan] requantisation scales
+        float* dump;          // FP32 forms: |Y|^2 summed over each K-block's frames
+                              // [n_in][n_int / tb][n_chan], or nullptr
+    };
     void* spec;            // spectra in the K-block layout
     float* beams;          // [2][n_int][n_chan] raw-resolution beams (0 inc, 1 coh)
     const float2* tw;      // FFT twiddles laid out as fengine_tw_angle() describes
@@ -163,10 +167,10 @@ cudaError_t launch_phasor_setup(int n_ant, int n_chan, int n_fft, int n_int, int
                                 const double* phi0, const double* rate, float2* pf, float2* ff, int* D,
                                 cudaStream_t s, const int64_t* g0_dev = nullptr);
 
-// Auto-power dumps from the FP32 K-block spectra (quad: the channel-quad layout): P[i][d][k] = sum
-// of |Y_i[t][k]|^2 over the `dump` frames of dump d (dump a multiple of tb_fp32(n_chan) dividing n_int).
-cudaError_t launch_power_dumps(const float* spec, int n_in, int n_chan, int n_int, int dump, float* P,
-                               cudaStream_t s, bool quad = false);
+// Auto-power dumps from the F-engine's K-block sums (FeParams::dump, [n_in][n_int / tb][n_chan], tb =
+// tb_fp32(n_chan)): P[i][d][k] = sum of |Y_i[t][k]|^2 over the `dump` frames of dump d, dump a
+// multiple of tb dividing n_int (with dump = tb the sums are the dumps, and nothing is launched).
+cudaError_t launch_power_dumps(const float* part, int n_in, int n_chan, int n_int, int dump, float* P, cudaStream_t s);
 
 // Time-domain voltage blanker (blank.cu, Sec. 5, Eq. 3-4) on rows x[i][0..n) cut into blocks of
 // `block` samples (a multiple of 16): per block, stats [n_in][ceil(n / block)][4] = 2 med, 4 MAD,

@@ -361,9 +361,12 @@ __device__ __forceinline__ void fengine_cta(const FeParams& p, int block, FeCtl&
             const float2 w = wa[chs[c]];
             const float2 wx = make_float2(w.x, w.x), wy = make_float2(w.y, w.y), nwy = make_float2(-w.y, -w.y);
             const float2 g22 = make_float2(g2, g2);
+            float2 pw4 = make_float2(0.0f, 0.0f);      // |Y|^2 over this thread's frames (even, odd)
 #pragma unroll
             for (int j = 0; j < LP; ++j) {
-                incr[j][c] = __ffma2_rn(g22, __ffma2_rn(yr[j], yr[j], __fmul2_rn(yi[j], yi[j])), incr[j][c]);
+                const float2 pw = __ffma2_rn(yr[j], yr[j], __fmul2_rn(yi[j], yi[j]));
+                incr[j][c] = __ffma2_rn(g22, pw, incr[j][c]);
+                if constexpr (MODE == OUT_FP32) pw4 = j ? __fadd2_rn(pw4, pw) : pw;
                 if (a == 0) {
                     cre[j][c] = make_float2(0.0f, 0.0f);
                     cim[j][c] = make_float2(0.0f, 0.0f);
@@ -382,6 +385,7 @@ __device__ __forceinline__ void fengine_cta(const FeParams& p, int block, FeCtl&
             }
             const int64_t blk = (static_cast<int64_t>(chs[c]) * ntb + kb_run) * blk_elems;
             if constexpr (MODE == OUT_FP32) {
+                if (p.dump) p.dump[(static_cast<int64_t>(i) * ntb + kb_run) * M + chs[c]] = pw4.x + pw4.y;
                 // 4-frame K-blocks: one 32-byte piece per (channel, input), rows 2i and 2i + 1 as
                 // neighbouring granules, in the order the XOR placement of row group G gives them
                 const int G = (2 * i) >> 3;

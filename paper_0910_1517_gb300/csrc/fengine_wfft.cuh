@@ -85,7 +85,9 @@ struct WCtl {
     int Ds[kMaxAnt];
 };
 
-template <int M, int MODE>
+// DUMP: also the K-block power sums (FeParams::dump).  An instantiation of its own: as a run-time branch
+// it spilled and took the GMRT-scale FP32 form without dumps from 1.58 to 1.62 ms.
+template <int M, int MODE, bool DUMP>
 __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams p) {
     using P = WPlan<M>;
     using S = WSmem<M>;
@@ -324,6 +326,12 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
                     cre[j][c] = __ffma2_rn(nwy, yi[j], __ffma2_rn(wx, yr[j], cre[j][c]));
                     cim[j][c] = __ffma2_rn(wy, yr[j], __ffma2_rn(wx, yi[j], cim[j][c]));
                 }
+                if constexpr (DUMP) {          // the power dumps' 8-frame sums, channels consecutive across lanes
+                    float2 pw = make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int j = 0; j < LP; ++j) pw = __ffma2_rn(yr[j], yr[j], __ffma2_rn(yi[j], yi[j], pw));
+                    if (live) p.dump[(static_cast<int64_t>(i) * ntb + kb_run) * M + chs[c]] = pw.x + pw.y;
+                }
                 if (detect) {                  // detect, add the polarisations, start the next sum
 #pragma unroll
                     for (int j = 0; j < LP; ++j) {
@@ -489,22 +497,24 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
     }
 }
 
-template <int M, int MODE>
+template <int M, int MODE, bool DUMP = false>
 cudaError_t launch_w(const FeParams& p, cudaStream_t s) {
+    if constexpr (!DUMP && (MODE == OUT_FP32 || MODE == OUT_F32Q))   // the forms that can dump powers
+        if (p.dump) return launch_w<M, MODE, true>(p, s);
     using P = WPlan<M>;
     const size_t smem = WSmem<M>::total;
     // the register split (setmaxnreg) hands the FFT group's registers to the epilogue group: it
     // needs exactly the 512 x 128 registers of the launch, or the epilogue warps would wait for
     // registers that never come -- refuse to launch otherwise
     cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, fengine_w_kernel<M, MODE>);
+    cudaError_t e = cudaFuncGetAttributes(&fa, fengine_w_kernel<M, MODE, DUMP>);
     if (e != cudaSuccess) return e;
     if (fa.numRegs != kWRegs) return cudaErrorInvalidConfiguration;
-    e = cudaFuncSetAttribute(fengine_w_kernel<M, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(fengine_w_kernel<M, MODE, DUMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     const int grid = (p.n_int + P::F - 1) / P::F;
-    fengine_w_kernel<M, MODE><<<grid, kWThreads, smem, s>>>(p);
+    fengine_w_kernel<M, MODE, DUMP><<<grid, kWThreads, smem, s>>>(p);
     return cudaGetLastError();
 }
 

@@ -82,6 +82,7 @@ struct corr {
     // auto-power dumps for the RFI stage (0 = off)
     int dump = 0;
     float* d_power = nullptr;
+    float* d_dump_part = nullptr;        // the F-engine's K-block sums (d_power itself when a dump is one K-block)
     // time-domain voltage blanker (Sec. 5, Eq. 3-4; blank_M = 0: off): blocks of 2^blank_log2 samples,
     // noise table [n_in][noise_L], per-block statistics [n_in][blank_nb][4] of the last integration
     // (blank_cap blocks per input allocated), covering blank_n samples of each row

@@ -187,7 +187,7 @@ extern "C" int corr_integrate_static(int n_ant, int n_pol, int n_fft, int n_int,
     fp.ff = reinterpret_cast<const float2*>(base + L.ff);
     fp.wcoh = reinterpret_cast<const float2*>(base + L.wcoh);
     fp.ginc = reinterpret_cast<const float*>(base + L.ginc);
-    fp.scale = nullptr;
+    fp.dump = nullptr;
     fp.spec = base + L.spec;
     fp.beams = beams;
     fp.tw = reinterpret_cast<const float2*>(base + L.tw);
