@@ -200,7 +200,8 @@ int gbx::run_integration(corr* h, const int8_t* x, int64_t ld, int64_t n_avail, 
         h->blank_nb = nb;
         h->blank_n = need;
     }
-    CU(launch_fengine(fp, fmode, s));
+    if (h->fe_split.parts > 1) CU(launch_fengine_split(fp, fmode, h->fe_split, s));
+    else CU(launch_fengine(fp, fmode, s));
     if (int rc = mark(h, 2, s)) return rc;
     XParams xp{};
     xp.spec = h->d_spec;
@@ -498,6 +499,11 @@ int corr_create(corr_t** out, int n_ant, int n_pol, int n_fft, int n_int) {
     CUB(cudaMemset(h->d_vis, 0, nvis * sizeof(float2)));
     CUB(cudaMemset(h->d_vis_int, 0, nvis * sizeof(int2)));
     CUB(cudaMemset(h->d_scale, 0, ni * nch * sizeof(float)));
+    h->fe_split = fe_plan(n_ant, n_pol, h->n_chan, n_int, h->n_sm);
+    if (h->fe_split.parts > 1) {
+        CUB(dalloc(&h->d_fe_part, fe_split_floats(h->fe_split, n_pol, h->n_chan)));
+        h->fe_split = fe_split_in(h->fe_split, h->d_fe_part, h->n_chan);
+    }
     CUB(dalloc(&h->d_tw, static_cast<size_t>(fengine_tw_count(n_fft))));
     CUB(launch_fengine_twiddles(n_fft, h->d_tw, h->stream));
     CUB(cudaStreamSynchronize(h->stream));
@@ -548,7 +554,7 @@ int corr_destroy(corr_t* h) {
         cudaFree(h->vis_b[1]);
     }
     if (h->xtab_b1) cudaFree(h->xtab_b1);
-    void* bufs[] = {h->d_ring, h->d_ring2, h->d_model, h->d_pf, h->d_ff, h->d_D, h->d_wcoh, h->d_ginc, h->d_scale,
+    void* bufs[] = {h->d_fe_part, h->d_ring, h->d_ring2, h->d_model, h->d_pf, h->d_ff, h->d_D, h->d_wcoh, h->d_ginc, h->d_scale,
                     h->d_tw, h->d_spec, h->d_beams_raw, h->d_vis, h->d_vis_part, h->d_vis_int, h->d_err};
     for (void* b : bufs)
         if (b) cudaFree(b);

@@ -85,10 +85,10 @@ cudaError_t launch_fengine_twiddles(int n_fft, float2* tw, cudaStream_t s) {
 cudaError_t launch_fengine(const FeParams& p, int mode, cudaStream_t s) {
     if (p.n_chan * 2 != p.n_fft) return cudaErrorInvalidValue;
     switch (mode) {
-        case OUT_FP32: return launch_w_mode<OUT_FP32>(p, s);
-        case OUT_F16: return launch_w_mode<OUT_F16>(p, s);
-        case OUT_F32Q: return launch_w_mode<OUT_F32Q>(p, s);
-        case OUT_I8B: return launch_w_mode<OUT_I8B>(p, s);
+        case OUT_FP32: return launch_w_mode<OUT_FP32, false>(p, s, nullptr);
+        case OUT_F16: return launch_w_mode<OUT_F16, false>(p, s, nullptr);
+        case OUT_F32Q: return launch_w_mode<OUT_F32Q, false>(p, s, nullptr);
+        case OUT_I8B: return launch_w_mode<OUT_I8B, false>(p, s, nullptr);
         default: return cudaErrorInvalidValue;
     }
 }

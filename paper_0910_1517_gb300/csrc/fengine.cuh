@@ -158,6 +158,27 @@ __device__ inline float2 model_fringe_phasor(double phi0, double rate, int64_t g
 }
 
 cudaError_t launch_fengine(const FeParams& p, int mode, cudaStream_t s);
+
+// Frame blocks shared by several CTAs (n_chan <= 1024).  A CTA walks every input of its frame block, so
+// an integration takes whole rounds of the SMs: 2 blocks of a tiny one leave 150 idle, 512 blocks on
+// 152 SMs take four rounds for 3.4.  The blocks of the last, partial round are therefore cut into
+// `parts` CTAs that take n_ant / parts antennas each, where that shortens the launch (fe_plan, by
+// more than 6 % of the whole); their beam sums go to inc [parts][frames][n_chan] and coh
+// [parts][n_pol][frames][n_chan], from where one kernel adds them.  Measured, whole integrations:
+// 4 antennas x 64 spectra of 512 points 64 -> 49 us (2 blocks, 4 parts), 60 antennas x 160 of 256
+// points 484 -> 103 us (3 blocks), 16 antennas x 1488 of 2048 points 460 -> 325 us (186 blocks, 34
+// of them shared), 32 antennas x 4096 behind the blanker 1.76 -> 1.66 ms (512 blocks, 56 shared).
+struct FeSplit {
+    int full = 0;          // blocks of the full rounds: whole CTAs, the first ones
+    int parts = 0;         // CTAs a block after them (0 or 1: nothing is shared)
+    int frames = 0;        // frames of the shared blocks
+    float* inc = nullptr;
+    float2* coh = nullptr;
+};
+FeSplit fe_plan(int n_ant, int n_pol, int n_chan, int n_int, int n_sm);     // without buffers
+size_t fe_split_floats(const FeSplit& sp, int n_pol, int n_chan);           // floats of its buffers
+FeSplit fe_split_in(FeSplit sp, float* buf, int n_chan);                     // ... placed at buf (16-byte aligned)
+cudaError_t launch_fengine_split(const FeParams& p, int mode, const FeSplit& sp, cudaStream_t s);
 // true where launch_fengine launches 2-CTA clusters (n_chan 2048, fp16 layouts and int8 bytes)
 bool fengine_clustered(int n_chan, int mode);
 

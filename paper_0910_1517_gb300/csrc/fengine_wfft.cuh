@@ -22,6 +22,8 @@
 //     both groups, and the copies still in flight are waited for before the CTA exits.
 #pragma once
 
+#include <type_traits>
+
 #include "fengine_impl.cuh"
 
 namespace gbx {
@@ -87,8 +89,17 @@ struct WCtl {
 
 // DUMP: also the K-block power sums (FeParams::dump).  An instantiation of its own: as a run-time branch
 // it spilled and took the GMRT-scale FP32 form without dumps from 1.58 to 1.62 ms.
-template <int M, int MODE, bool DUMP>
-__global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams p) {
+// SPLIT: the CTAs from p.sp.full on share frame blocks, p.sp.parts to a block, each walking its own
+// antennas and leaving its beam sums in p.sp (fe_plan); also an instantiation of its own (extra
+// registers spill at 1024 points).
+struct FeParamsSplit : FeParams {
+    FeSplit sp;
+};
+template <bool SPLIT>
+using FeParamsOf = typename std::conditional<SPLIT, FeParamsSplit, FeParams>::type;
+
+template <int M, int MODE, bool DUMP, bool SPLIT>
+__global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParamsOf<SPLIT> p) {
     using P = WPlan<M>;
     using S = WSmem<M>;
     constexpr int PP = P::P, G = P::G, F = P::F, N = P::N, L = P::L;
@@ -105,9 +116,22 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
     volatile int* abort_flag = &ctl.abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int t0 = blockIdx.x * F;
+    // this CTA's frame block, and with SPLIT its antennas a0 .. a0 + na_ - 1 (part < 0: all of them)
+    int part = -1, a0 = 0, na_ = 0, block = blockIdx.x;
+    if constexpr (SPLIT) {
+        na_ = p.n_ant;
+        if (block >= p.sp.full) {
+            part = (block - p.sp.full) % p.sp.parts;
+            block = p.sp.full + (block - p.sp.full) / p.sp.parts;
+            a0 = part * p.n_ant / p.sp.parts;
+            na_ = (part + 1) * p.n_ant / p.sp.parts - a0;
+        }
+    }
+    const int t0 = block * F;
     const int n_fr = min(F, p.n_int - t0);
-    const int n_iter = p.n_in;                // polarisation-major: it = pol * n_ant + a
+    const int n_iter = SPLIT ? na_ * p.n_pol : p.n_in;        // polarisation-major: it = pol * n_ant + a
+    auto pol_of = [&](int it) { return it / (SPLIT ? na_ : p.n_ant); };
+    auto ant_of = [&](int it) { return SPLIT ? a0 + it % na_ : it % p.n_ant; };
 
     const float2* twsrc = p.tw + fengine_tw_wfft_offset(N);
     for (int m = tid; m < S::kTw1 + S::kTwN; m += kWThreads) tw1[m] = twsrc[m];
@@ -131,7 +155,7 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
         // integer delay); bytes past the last 16-byte boundary are copied by the lanes only when
         // rounding the copy up would read past the row's readable samples
         auto issue = [&](int it) {
-            const int pol = it / p.n_ant, a = it % p.n_ant;
+            const int pol = pol_of(it), a = ant_of(it);
             const int i = a * p.n_pol + pol;
             unsigned char* dst = stage0 + (it & 1) * P::STAGE;
             const int64_t s0 = static_cast<int64_t>(t0) * N + ctl.Ds[a];
@@ -152,7 +176,7 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
         // phasor, beam-weight and fringe rows of the antenna of input `it` (n_fr * 8 bytes of
         // fringe phasors: a multiple of 16 since n_fr is a multiple of 16 or F)
         auto issue_tab = [&](int it) {
-            const int a = it % p.n_ant;
+            const int a = ant_of(it);
             float2* dst = tab + (it & 1) * S::kTab;
             uint64_t* tb = &ctl.tbar[it & 1];
             fence_proxy_async_smem();
@@ -183,7 +207,7 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
             // a timed-out wait stops the CTA at the next barrier; this pass runs on whatever the
             // buffers hold (every address is data-independent), so no thread leaves the group alone
             if (!ok) *abort_flag = 1;
-            const int a = it % p.n_ant;
+            const int a = ant_of(it);
             const int64_t s0 = static_cast<int64_t>(t0) * N + ctl.Ds[a];
             float2* Rw = Xbuf + b * (kWFftWarps * P::REG) + warp * P::REG;   // this warp's region
             // ---- pass 1: lane = column l of each of the warp's G frames, P-point DFTs
@@ -288,7 +312,7 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
             }
         for (int it = 0; it < n_iter; ++it) {
             const int b = it & 1;
-            const int pol = it / p.n_ant, a = it % p.n_ant;
+            const int pol = pol_of(it), a = ant_of(it);
             const int i = a * p.n_pol + pol;
             const float g2 = p.ginc[a];
             const float2 g22 = make_float2(g2, g2);
@@ -309,7 +333,7 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
             const float2* pfa = tab + b * S::kTab;
             const float2* wa = pfa + M;
             const float2* fra = pfa + 2 * M;   // fringe phasors of the CTA's frames
-            const bool detect = a == p.n_ant - 1;   // this polarisation's coherent sums are complete
+            const bool detect = a == (SPLIT ? a0 + na_ : p.n_ant) - 1;   // this polarisation's coherent sums are complete
             // every lane computes (the FP32 stores trade values between lanes, and `live` is not
             // warp-uniform when a warp spans several frame groups); only live lanes write
             constexpr int PG = TB / 2;
@@ -335,6 +359,18 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
                 if (detect) {                  // detect, add the polarisations, start the next sum
 #pragma unroll
                     for (int j = 0; j < LP; ++j) {
+                        if constexpr (SPLIT) {
+                            if (part >= 0) {           // a part's voltage sums
+                                if (live) {
+                                    float2* q = p.sp.coh + ((static_cast<int64_t>(part) * p.n_pol + pol) * p.sp.frames + (t0 - p.sp.full * F) + fg * L + 2 * j) * M + chs[c];
+                                    q[0] = make_float2(cre[j][c].x, cim[j][c].x);
+                                    q[M] = make_float2(cre[j][c].y, cim[j][c].y);
+                                }
+                                cre[j][c] = make_float2(0.0f, 0.0f);
+                                cim[j][c] = make_float2(0.0f, 0.0f);
+                                continue;
+                            }
+                        }
                         const float2 pw = __ffma2_rn(cim[j][c], cim[j][c], __fmul2_rn(cre[j][c], cre[j][c]));
                         cre[j][c] = make_float2(0.0f, 0.0f);
                         cim[j][c] = make_float2(0.0f, 0.0f);
@@ -488,62 +524,62 @@ __global__ void __launch_bounds__(kWThreads, 1) fengine_w_kernel(const FeParams 
         }
         // incoherent beam of this thread's points
         if (!*abort_flag && live) {
+            float* inc = p.beams;
+            if constexpr (SPLIT)
+                if (part >= 0) inc = p.sp.inc + (static_cast<int64_t>(part) * p.sp.frames - p.sp.full * F) * M;
 #pragma unroll
             for (int l = 0; l < L; ++l)
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    p.beams[static_cast<int64_t>(t0 + fg * L + l) * M + chs[c]] = (l & 1) ? incr[l >> 1][c].y : incr[l >> 1][c].x;
+                    inc[static_cast<int64_t>(t0 + fg * L + l) * M + chs[c]] = (l & 1) ? incr[l >> 1][c].y : incr[l >> 1][c].x;
         }
     }
 }
 
-template <int M, int MODE, bool DUMP = false>
-cudaError_t launch_w(const FeParams& p, cudaStream_t s) {
+template <int M, int MODE, bool SPLIT, bool DUMP = false>
+cudaError_t launch_w(const FeParams& p, cudaStream_t s, const FeSplit* sp) {
     if constexpr (!DUMP && (MODE == OUT_FP32 || MODE == OUT_F32Q))   // the forms that can dump powers
-        if (p.dump) return launch_w<M, MODE, true>(p, s);
+        if (p.dump) return launch_w<M, MODE, SPLIT, true>(p, s, sp);
+    auto kern = fengine_w_kernel<M, MODE, DUMP, SPLIT>;
     using P = WPlan<M>;
     const size_t smem = WSmem<M>::total;
     // the register split (setmaxnreg) hands the FFT group's registers to the epilogue group: it
     // needs exactly the 512 x 128 registers of the launch, or the epilogue warps would wait for
     // registers that never come -- refuse to launch otherwise
     cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, fengine_w_kernel<M, MODE, DUMP>);
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
     if (e != cudaSuccess) return e;
     if (fa.numRegs != kWRegs) return cudaErrorInvalidConfiguration;
-    e = cudaFuncSetAttribute(fengine_w_kernel<M, MODE, DUMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    const int grid = (p.n_int + P::F - 1) / P::F;
-    fengine_w_kernel<M, MODE, DUMP><<<grid, kWThreads, smem, s>>>(p);
+    const int blocks = (p.n_int + P::F - 1) / P::F;
+    if constexpr (SPLIT) {
+        const int grid = sp->full + (blocks - sp->full) * sp->parts;
+        FeParamsSplit q;
+        static_cast<FeParams&>(q) = p;
+        q.sp = *sp;
+        kern<<<grid, kWThreads, smem, s>>>(q);
+    } else {
+        kern<<<blocks, kWThreads, smem, s>>>(p);
+    }
     return cudaGetLastError();
 }
 
-template <int MODE>
-cudaError_t launch_w_mode(const FeParams& p, cudaStream_t s) {
-    if constexpr (MODE == OUT_F32Q || MODE == OUT_I8B) {   // n_chan 32 .. 1024 (int8 bytes: .. 2048)
-        switch (p.n_chan) {
-            case 32: return launch_w<32, MODE>(p, s);
-            case 64: return launch_w<64, MODE>(p, s);
-            case 128: return launch_w<128, MODE>(p, s);
-            case 256: return launch_w<256, MODE>(p, s);
-            case 512: return launch_w<512, MODE>(p, s);
-            case 1024: return launch_w<1024, MODE>(p, s);
-            case 2048:   // 4-frame CTAs in cluster pairs: the kernel of fengine_impl.cuh
-                if constexpr (MODE == OUT_I8B) return launch_t<2048, MODE>(p, s);
-                return cudaErrorInvalidValue;
-            default: return cudaErrorInvalidValue;
-        }
-    } else {
+// The launch for p.n_chan; SPLIT only below 2048 channels
+template <int MODE, bool SPLIT>
+cudaError_t launch_w_mode(const FeParams& p, cudaStream_t s, const FeSplit* sp) {
     switch (p.n_chan) {
-        case 32: return launch_w<32, MODE>(p, s);
-        case 64: return launch_w<64, MODE>(p, s);
-        case 128: return launch_w<128, MODE>(p, s);
-        case 256: return launch_w<256, MODE>(p, s);
-        case 512: return launch_w<512, MODE>(p, s);
-        case 1024: return launch_w<1024, MODE>(p, s);
-        case 2048: return launch_t<2048, MODE>(p, s);   // 4-frame CTAs: the kernel of fengine_impl.cuh
+        case 32: return launch_w<32, MODE, SPLIT>(p, s, sp);
+        case 64: return launch_w<64, MODE, SPLIT>(p, s, sp);
+        case 128: return launch_w<128, MODE, SPLIT>(p, s, sp);
+        case 256: return launch_w<256, MODE, SPLIT>(p, s, sp);
+        case 512: return launch_w<512, MODE, SPLIT>(p, s, sp);
+        case 1024: return launch_w<1024, MODE, SPLIT>(p, s, sp);
+        case 2048:   // 4-frame CTAs: the kernel of fengine_impl.cuh (which writes no channel quads of FP32)
+            if constexpr (!SPLIT && MODE != OUT_F32Q) return launch_t<2048, MODE>(p, s);
+            return cudaErrorInvalidValue;
         default: return cudaErrorInvalidValue;
-    }
     }
 }
 

@@ -63,6 +63,8 @@ struct corr {
     float* d_ginc = nullptr;
     float* d_scale = nullptr;
     float2* d_tw = nullptr;
+    gbx::FeSplit fe_split;               // frame blocks the F-engine shares among CTAs (single integrations)
+    float* d_fe_part = nullptr;          // ... and their partial beam sums
     void* d_spec = nullptr;
     float* d_beams_raw = nullptr;
     float* d_beams = nullptr;

@@ -51,6 +51,7 @@ size_t align256(size_t v) { return (v + 255) & ~static_cast<size_t>(255); }
 
 struct Layout {
     size_t err, D, ginc, pf, wcoh, ff, tw, spec, total;
+    size_t part;                  // partial beam sums of shared frame blocks, if they fit after the rest
 };
 
 Layout layout(int n_ant, int n_pol, int n_fft, int n_int) {
@@ -73,7 +74,7 @@ Layout layout(int n_ant, int n_pol, int n_fft, int n_int) {
     o = align256(o + sizeof(float2) * gbx::fengine_tw_count(n_fft));
     L.spec = o;
     o = align256(o + sizeof(float) * nch * static_cast<size_t>(n_int) * gbx::rows_fp32(n_ant * n_pol));
-    L.total = o;
+    L.total = L.part = o;
     return L;
 }
 
@@ -192,7 +193,11 @@ extern "C" int corr_integrate_static(int n_ant, int n_pol, int n_fft, int n_int,
     fp.beams = beams;
     fp.tw = reinterpret_cast<const float2*>(base + L.tw);
     fp.err = reinterpret_cast<unsigned*>(base + L.err);
-    if (gbx::launch_fengine(fp, gbx::OUT_FP32, s) != cudaSuccess)
+    gbx::FeSplit sp = gbx::fe_plan(n_ant, n_pol, fp.n_chan, n_int, n_sm);
+    const size_t part_bytes = sizeof(float) * gbx::fe_split_floats(sp, n_pol, fp.n_chan);
+    const bool shared = sp.parts > 1 && L.part + part_bytes <= kScratchBytes;
+    if (shared) sp = gbx::fe_split_in(sp, reinterpret_cast<float*>(base + L.part), fp.n_chan);
+    if ((shared ? gbx::launch_fengine_split(fp, gbx::OUT_FP32, sp, s) : gbx::launch_fengine(fp, gbx::OUT_FP32, s)) != cudaSuccess)
         return fail(CORR_E_CUDA, "corr_integrate_static: F-engine launch");
     gbx::XParams xp{};
     xp.spec = base + L.spec;
