@@ -39,6 +39,7 @@ struct alignas(128) XtSub {   // (the tensor map's own alignment)
     // stage is one TMA copy through this 5-D tensor map over (16 floats, channel in quad, input,
     // K-block, quad), box (16, 1, n_in, ks / 8, 1); it lands [kb][2 n_in rows][8 frames]
     CUtensorMap tmap;
+    CUtensorMap tmap_hi;   // the same over inputs 64 .. n_in - 1, for the second item of a Gram of over 128 rows
     int quad;
     const __half* spec;    // [k][kb][2 n_in][8] fp16 K-block layout
     // in8 = 1: spec holds the same layout in int8 bytes (rows of 8 bytes, the F-engine's OUT_I8B);

@@ -12,7 +12,7 @@
 // Work items are (sub-array, channel, row block): 128 Gram rows a0..a0+127 against
 // columns b0..b0+N-1.  Up to 128 rows need one item (N <= 128, the rest of the 128
 // rows is ignored); 256 rows need two (rows 0-127 x columns 0-255, rows 128-255 x
-// columns 128-255).  A persistent CTA walks a cost-ordered item list; several
+// columns 128-255; gathered by TMA, the second's stages hold its rows alone).  A persistent CTA walks a cost-ordered item list; several
 // sub-arrays of different sizes share one launch.
 //
 // Roles: warp 0 streams stages in (and owns the TMEM allocation), warp 1 issues
@@ -133,6 +133,7 @@ struct Shared {
 };
 
 struct ItemGeo {
+    int base;      // Gram row and column of the stage's first (a second item gathered by TMA has its own rows only)
     int sub, k, a0, b0, N, R, ntb, n_stage, n_chunk, nkb_stage;
     int Rp, tb32, ntb32;   // FP32 form: padded rows, frames per FP32 K-block, FP32 K-blocks per channel
     bool dbl;      // N <= 128: rotating 128-column accumulators
@@ -150,7 +151,14 @@ __device__ __forceinline__ ItemGeo item_geo(const XtBatch& t, int it) {
     g.k = e.y;
     const XtSub& s = t.sub[g.sub];
     g.R = 2 * s.n_in;
+    const bool paired = g.R == 128;
+    g.base = 0;
     g.a0 = 128 * e.z;
+    if (e.z && (s.quad || s.in8)) {   // the stage holds these rows alone
+        g.base = 128;
+        g.R -= 128;
+        g.a0 = 0;
+    }
     g.b0 = (g.R > 128) ? g.a0 : 0;
     g.N = ((g.R - g.b0 + 15) / 16) * 16;
     g.Rp = rows_fp32(s.n_in);
@@ -158,7 +166,7 @@ __device__ __forceinline__ ItemGeo item_geo(const XtBatch& t, int it) {
     g.ntb32 = s.n_int / g.tb32;
     g.dbl = g.N <= 128;
     g.sep = g.dbl && (s.spec32 != nullptr || s.in8);
-    g.pair = g.sep && s.spec32 != nullptr && g.R == 128;
+    g.pair = g.sep && s.spec32 != nullptr && paired;
     g.cross = g.sep && s.spec32 != nullptr && !g.pair;
     g.nbuf = !g.dbl ? 1 : (g.sep && s.spec32 != nullptr ? 2 : kAccBufs);
     g.ntb = s.n_int / kTbHalf;
@@ -206,7 +214,7 @@ __device__ __forceinline__ void write_piece(const XtSub& s, const ItemGeo& ig, i
     for (int jh = 0; jh < W / 4; ++jh) {
         const uint32_t r0 = __shfl_xor_sync(0xffffffffu, odd ? run[2 * jh] : run[2 * jh + H], 1);
         const uint32_t r1 = __shfl_xor_sync(0xffffffffu, odd ? run[2 * jh + 1] : run[2 * jh + H + 1], 1);
-        const int j = ((ig.b0 + j0) >> 1) + jh + (odd ? W / 4 : 0);
+        const int j = ((ig.base + ig.b0 + j0) >> 1) + jh + (odd ? W / 4 : 0);
         // G[2i][2j], G[2i][2j+1], G[2i+1][2j], G[2i+1][2j+1]
         const uint32_t g_r0c0 = odd ? r0 : run[2 * jh];
         const uint32_t g_r0c1 = odd ? r1 : run[2 * jh + 1];
@@ -444,9 +452,8 @@ __device__ __forceinline__ void split_pair(float2 w, float2 sc, float2 nsc, floa
 // the converter threads (a stage has at most kUnits per thread, so that a thread first loads all
 // its units, while the operand slot may still be read by the tensor core, then converts and stores
 // them: their latencies overlap, and none is left of a remainder loop):
-//   int8 bytes [kb][R rows][8 frames]: unit (j, r), 8 bytes, becomes the 16-byte row r of K-block j
-//     of the fp16 operand tile.  Only rows b0 .. R - 1 are converted: the second item of a 256-row
-//     Gram (rows and columns 128 .. R - 1) reads no others.
+//   int8 bytes [kb][R rows][8 frames]: unit u = j R + r, 8 bytes, becomes the 16-byte row r of K-block
+//     j of the fp16 operand tile
 //   FP32, channel-quad stage [kb][R rows][8 frames]: unit u = (j R + r) 2 + h, frames 4h .. 4h + 3 of
 //     row r in K-block j (one 16-byte load; consecutive units, consecutive bytes), whose hi and lo
 //     halves (8 bytes each) go into row r of K-block j of the two operand tiles
@@ -475,10 +482,10 @@ __device__ __forceinline__ void convert_stages(const XtBatch& t, Shared& sh, uns
         const float2 sc = make_float2(s.split_scale, s.split_scale), nsc = make_float2(-sc.x, -sc.x);
         const float2 k8 = make_float2(8193.0f * sc.x, 8193.0f * sc.x);
         const int lo_off = kPairs ? 2048 : ig.nkb_stage * R * 16;
-        const bool quad = s.quad, part = ig.b0 != 0;
-        const int Rs = kIn8 ? R - ig.b0 : R, n_int = s.n_int, ks = s.ks;   // rows converted of a K-block
+        const bool quad = s.quad;
+        const int n_int = s.n_int, ks = s.ks;
         // unit ct of a stage as (K-block j0, row r0), and the step of kConvThreads units
-        const int r0 = ct % Rs, j0 = ct / Rs, dr = kConvThreads % Rs, dj = kConvThreads / Rs;
+        const int r0 = ct % R, j0 = ct / R, dr = kConvThreads % R, dj = kConvThreads / R;
         for (int st = 0; st < ig.n_stage; ++st, ++g) {
             const int fs = g % nin, os = g % nop;
             auto wait = [&](uint64_t* bar, uint32_t parity, unsigned bit) {
@@ -494,30 +501,14 @@ __device__ __forceinline__ void convert_stages(const XtBatch& t, Shared& sh, uns
             unsigned char* dst = smem + os * kSlot2;
             if constexpr (kIn8) {
                 uint2 q[kUnits];
-                const int units = kbs * Rs;
-                if (!part) {
+                const int units = kbs * R;
 #pragma unroll
-                    for (int i = 0; i < kUnits; ++i) {
-                        const int u = ct + i * kConvThreads;
-                        q[i] = u < units ? *reinterpret_cast<const uint2*>(src + 8 * u) : make_uint2(0u, 0u);
-                    }
-                } else {
-                    int r = r0, j = j0;
-#pragma unroll
-                    for (int i = 0; i < kUnits; ++i) {
-                        q[i] = ct + i * kConvThreads < units ? *reinterpret_cast<const uint2*>(src + 8 * (j * R + ig.b0 + r))
-                                                             : make_uint2(0u, 0u);
-                        r += dr;
-                        j += dj;
-                        if (r >= Rs) {
-                            r -= Rs;
-                            ++j;
-                        }
-                    }
+                for (int i = 0; i < kUnits; ++i) {
+                    const int u = ct + i * kConvThreads;
+                    q[i] = u < units ? *reinterpret_cast<const uint2*>(src + 8 * u) : make_uint2(0u, 0u);
                 }
                 if (!wait_op()) return;
                 const __half2 bias = __float2half2_rn(1152.0f);
-                int r = r0, j = j0;
 #pragma unroll
                 for (int i = 0; i < kUnits; ++i) {
                     const uint32_t x[2] = {q[i].x ^ 0x80808080u, q[i].y ^ 0x80808080u};
@@ -528,16 +519,8 @@ __device__ __forceinline__ void convert_stages(const XtBatch& t, Shared& sh, uns
                         const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&hb), bias);
                         w[m] = *reinterpret_cast<const uint32_t*>(&v);
                     }
-                    const int u = part ? j * R + ig.b0 + r : ct + i * kConvThreads;
-                    if (ct + i * kConvThreads < units) *reinterpret_cast<uint4*>(dst + 16 * u) = make_uint4(w[0], w[1], w[2], w[3]);
-                    if (part) {
-                        r += dr;
-                        j += dj;
-                        if (r >= Rs) {
-                            r -= Rs;
-                            ++j;
-                        }
-                    }
+                    const int u = ct + i * kConvThreads;
+                    if (u < units) *reinterpret_cast<uint4*>(dst + 16 * u) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             } else if (quad) {
                 float4 q[kUnits];
@@ -566,7 +549,7 @@ __device__ __forceinline__ void convert_stages(const XtBatch& t, Shared& sh, uns
                 float4 q[kUnits8][2];
                 const int units = kbs * R;
                 {
-                    int r = r0, j = j0;              // (Rs is R here)
+                    int r = r0, j = j0;
 #pragma unroll
                     for (int i = 0; i < kUnits8; ++i) {
                         const bool sw = tb == 8 && ((r >> 2) & 1);
@@ -671,7 +654,7 @@ __global__ void __launch_bounds__((kForm != XT_FORM_F16 ? kWarps2 : kWarps1) * 3
         for (int it = blockIdx.x; it < t.n_items && go; it += gridDim.x) {
             const ItemGeo ig = item_geo(t, it);
             const XtSub& s = t.sub[ig.sub];
-            const int row = ig.a0 + lrow;
+            const int row = ig.base + ig.a0 + lrow;
             if (kForm == XT_FORM_F32 && ig.sep) {   // three products
                 for (int chunk = 0; chunk < ig.n_chunk; ++chunk, ++cc) {
                     const int b = cc % ig.nbuf;
@@ -753,17 +736,19 @@ __global__ void __launch_bounds__((kForm != XT_FORM_F16 ? kWarps2 : kWarps1) * 3
                     if (f32 && s.quad) {
                         // channel-quad layout: one 5-D tensor copy gathers the stage's pieces of channel k
                         // (a last, shorter stage reads zeros past the end and counts the whole box)
-                        if (st == 0) tmap_acquire(&s.tmap);
+                        const CUtensorMap* map = ig.base ? &s.tmap_hi : &s.tmap;
+                        if (st == 0) tmap_acquire(map);
                         const int nkb = s.ks / kTbHalf;
-                        mbar_arrive_expect_tx(&fullb[slot], static_cast<uint32_t>(nkb) * s.n_in * 64);
-                        tma_load_5d(dst, &s.tmap, 0, ig.k & 3, 0, st * nkb, ig.k >> 2, &fullb[slot]);
+                        mbar_arrive_expect_tx(&fullb[slot], static_cast<uint32_t>(nkb) * ig.R * 32);
+                        tma_load_5d(dst, map, 0, ig.k & 3, 0, st * nkb, ig.k >> 2, &fullb[slot]);
                     } else if (f32 && in8) {
                         // channel-quad int8 bytes: one 5-D tensor copy gathers the stage's 16-byte pieces
                         // of channel k into [kb][2 n_in rows][8 bytes] (half the fp16 bytes)
-                        if (st == 0) tmap_acquire(&s.tmap);
+                        const CUtensorMap* map = ig.base ? &s.tmap_hi : &s.tmap;
+                        if (st == 0) tmap_acquire(map);
                         const int nkb = s.ks / kTbHalf;
-                        mbar_arrive_expect_tx(&fullb[slot], static_cast<uint32_t>(nkb) * s.n_in * 16);
-                        tma_load_5d(dst, &s.tmap, 0, ig.k & 3, 0, st * nkb, ig.k >> 2, &fullb[slot]);
+                        mbar_arrive_expect_tx(&fullb[slot], static_cast<uint32_t>(nkb) * ig.R * 8);
+                        tma_load_5d(dst, map, 0, ig.k & 3, 0, st * nkb, ig.k >> 2, &fullb[slot]);
                     } else if (f32) {
                         // the stage's FP32 K-blocks of channel k are contiguous
                         const int frames = min(s.ks, s.n_int - st * s.ks);
@@ -917,15 +902,19 @@ bool xengine_tc_encode_quad(XtSub& x) {
         encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
     }
     const cuuint64_t ntb = static_cast<cuuint64_t>(x.n_int / kTbHalf);
-    const cuuint64_t dim[5] = {16, 4, static_cast<cuuint64_t>(x.n_in), ntb, static_cast<cuuint64_t>(x.n_chan / 4)};
     const cuuint64_t piece = b8 ? 16 : 64;         // bytes of one (channel, K-block, input) piece
     const cuuint64_t stride[4] = {piece, 4 * piece, 4 * piece * x.n_in, 4 * piece * x.n_in * ntb};   // bytes, dims 1..4
-    const cuuint32_t box[5] = {16, 1, static_cast<cuuint32_t>(x.n_in), static_cast<cuuint32_t>(x.ks / kTbHalf), 1};
     const cuuint32_t estride[5] = {1, 1, 1, 1, 1};
     void* base = b8 ? static_cast<void*>(const_cast<__half*>(x.spec)) : static_cast<void*>(const_cast<float*>(x.spec32));
-    return encode(&x.tmap, b8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, base, dim, stride, box, estride,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    auto map = [&](CUtensorMap* m, int first) {    // inputs first .. n_in - 1
+        const int n = x.n_in - first;
+        const cuuint64_t dim[5] = {16, 4, static_cast<cuuint64_t>(n), ntb, static_cast<cuuint64_t>(x.n_chan / 4)};
+        const cuuint32_t box[5] = {16, 1, static_cast<cuuint32_t>(n), static_cast<cuuint32_t>(x.ks / kTbHalf), 1};
+        return encode(m, b8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5,
+                      static_cast<char*>(base) + 4 * piece * first, dim, stride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    return map(&x.tmap, 0) && (x.n_in <= 64 || map(&x.tmap_hi, 64));
 }
 
 bool xengine_tc_supported(int n_in) { return n_in >= 1 && 2 * n_in <= 256; }
