@@ -203,6 +203,7 @@ int gbx::run_integration(corr* h, const int8_t* x, int64_t ld, int64_t n_avail, 
     if (h->fe_split.parts > 1) CU(launch_fengine_split(fp, fmode, h->fe_split, s));
     else CU(launch_fengine(fp, fmode, s));
     if (int rc = mark(h, 2, s)) return rc;
+    if (h->out_beams && h->beam_avg == 1) CU(cudaEventRecord(h->ev_beams, s));
     XParams xp{};
     xp.spec = h->d_spec;
     xp.n_ant = h->n_ant;
@@ -343,12 +344,17 @@ int enqueue_output(corr* h, int64_t index) {
     const size_t nb = 2 * static_cast<size_t>(h->n_int / h->beam_avg) * h->n_chan;
     h->slot_of[slot] = index;
     CU(cudaEventRecord(h->ev_int_done, h->stream));
+    auto copy_beams = [&]() {
+        return cudaMemcpyAsync(h->out_beams + nb * slot, h->beams_b[b], nb * sizeof(float), cudaMemcpyDeviceToHost, h->ostream);
+    };
+    if (h->out_beams && h->beam_avg == 1) {   // raw beams are the F-engine's
+        CU(cudaStreamWaitEvent(h->ostream, h->ev_beams, 0));
+        CU(copy_beams());
+    }
     CU(cudaStreamWaitEvent(h->ostream, h->ev_int_done, 0));
     CU(cudaMemcpyAsync(h->out_vis + nv * slot, h->vis_b[b], nv * sizeof(float), cudaMemcpyDeviceToHost,
                        h->ostream));
-    if (h->out_beams)
-        CU(cudaMemcpyAsync(h->out_beams + nb * slot, h->beams_b[b], nb * sizeof(float), cudaMemcpyDeviceToHost,
-                           h->ostream));
+    if (h->out_beams && h->beam_avg > 1) CU(copy_beams());
     CU(cudaEventRecord(h->ev_out[slot], h->ostream));
     CU(cudaEventRecord(h->ev_buf_free[b], h->ostream));
     return CORR_OK;
@@ -577,6 +583,7 @@ int corr_destroy(corr_t* h) {
     for (cudaEvent_t e : h->ev_model)
         if (e) cudaEventDestroy(e);
     if (h->ev_int_done) cudaEventDestroy(h->ev_int_done);
+    if (h->ev_beams) cudaEventDestroy(h->ev_beams);
     for (cudaEvent_t e : h->ev_buf_free)
         if (e) cudaEventDestroy(e);
     if (h->ostream) cudaStreamDestroy(h->ostream);
@@ -800,6 +807,7 @@ int corr_set_output_ring(corr_t* h, float* vis, float* beams, int n_slots) {
     if (!h->ostream) {
         CU(cudaStreamCreateWithFlags(&h->ostream, cudaStreamNonBlocking));
         CU(cudaEventCreateWithFlags(&h->ev_int_done, cudaEventDisableTiming));
+        CU(cudaEventCreateWithFlags(&h->ev_beams, cudaEventDisableTiming));
         for (cudaEvent_t& e : h->ev_buf_free) CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     }
     h->ev_out.resize(n_slots, nullptr);

@@ -47,6 +47,7 @@ struct corr {
     gbx::XtBatch* xtab_b1 = nullptr;     // tensor-core table naming buffer 1
     int out_buf = 0;
     cudaStream_t ostream = nullptr;
+    cudaEvent_t ev_beams = nullptr;      // raw beams complete (they leave while the X-engine runs)
     cudaEvent_t ev_int_done = nullptr, ev_buf_free[2] = {nullptr, nullptr};
     int batch_refs = 0;                  // batches (captured graphs) holding this handle's buffers
     // device tables and outputs
