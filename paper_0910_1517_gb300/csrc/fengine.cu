@@ -14,21 +14,10 @@ __global__ void phasor_setup_kernel(int n_ant, int n_chan, int n_fft, int n_int,
                                     const double* __restrict__ rate, float2* __restrict__ pf,
                                     float2* __restrict__ ff, int* __restrict__ D) {
     const int64_t g0 = g0_ptr ? *g0_ptr : g0_val;
-    const int64_t n1 = static_cast<int64_t>(n_ant) * n_chan, n2 = static_cast<int64_t>(n_ant) * n_int;
-    for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < n1 + n2 + n_ant;
-         q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        if (q < n1) {
-            const int a = static_cast<int>(q / n_chan), k = static_cast<int>(q % n_chan);
-            pf[q] = model_fstc_phasor(tau[a], k, n_fft);
-        } else if (q < n1 + n2) {
-            const int64_t r = q - n1;
-            const int a = static_cast<int>(r / n_int), t = static_cast<int>(r % n_int);
-            ff[r] = model_fringe_phasor(phi0[a], rate[a], g0 + t);
-        } else {
-            const int a = static_cast<int>(q - n1 - n2);
-            D[a] = model_int_delay(tau[a]);
-        }
-    }
+    const int64_t id = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (id < n_ant) D[id] = model_int_delay(tau[id]);
+    if (id / 32 < model_table_warps(n_ant, n_chan, n_int))
+        model_table(id / 32, n_ant, n_chan, n_fft, n_int, g0, tau, phi0, rate, pf, ff);
 }
 
 __global__ void twiddle_kernel(int n_fft, int count, float2* __restrict__ tw) {
@@ -100,9 +89,10 @@ bool fengine_clustered(int n_chan, int mode) {
 cudaError_t launch_phasor_setup(int n_ant, int n_chan, int n_fft, int n_int, int64_t g0, const double* tau,
                                 const double* phi0, const double* rate, float2* pf, float2* ff, int* D,
                                 cudaStream_t s, const int64_t* g0_dev) {
-    const int64_t total = static_cast<int64_t>(n_ant) * (n_chan + n_int) + n_ant;
-    const int grid = static_cast<int>(std::min<int64_t>((total + 255) / 256, 4096));
-    phasor_setup_kernel<<<grid, 256, 0, s>>>(n_ant, n_chan, n_fft, n_int, g0, g0_dev, tau, phi0, rate, pf, ff, D);
+    // 64 threads a block: two warps an SM from 152 warps on; at least one warp, so n_ant <= 128 delays too
+    const int64_t threads = std::max<int64_t>(32 * model_table_warps(n_ant, n_chan, n_int), n_ant);
+    phasor_setup_kernel<<<static_cast<unsigned>((threads + 63) / 64), 64, 0, s>>>(n_ant, n_chan, n_fft, n_int, g0, g0_dev, tau, phi0,
+                                                                                 rate, pf, ff, D);
     return cudaGetLastError();
 }
 

@@ -89,24 +89,15 @@ __global__ void static_tables_kernel(Model m, int n_ant, int n_fft, int n_int, i
     float2* pf = reinterpret_cast<float2*>(base + L.pf);
     float2* wcoh = reinterpret_cast<float2*>(base + L.wcoh);
     float2* ff = reinterpret_cast<float2*>(base + L.ff);
-    const int64_t n_pf = static_cast<int64_t>(n_ant) * M, n_ff = static_cast<int64_t>(n_ant) * n_int;
-    const int64_t total = n_pf + n_ff + n_ant;
-    for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < total;
-         q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        if (q < n_pf) {
-            const int a = static_cast<int>(q / M), k = static_cast<int>(q % M);
-            pf[q] = gbx::model_fstc_phasor(m.tau[a], k, n_fft);
-            wcoh[q] = make_float2(1.0f, 0.0f);
-        } else if (q < n_pf + n_ff) {
-            const int64_t r = q - n_pf;
-            const int a = static_cast<int>(r / n_int), t = static_cast<int>(r % n_int);
-            ff[r] = gbx::model_fringe_phasor(m.phi0[a], m.rate[a], g0 + t);
-        } else {
-            const int a = static_cast<int>(q - n_pf - n_ff);
-            D[a] = gbx::model_int_delay(m.tau[a]);
-            ginc[a] = 1.0f;
-        }
+    const int64_t id = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (id < n_ant) {
+        D[id] = gbx::model_int_delay(m.tau[id]);
+        ginc[id] = 1.0f;
     }
+    for (int64_t q = id; q < static_cast<int64_t>(n_ant) * M; q += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        wcoh[q] = make_float2(1.0f, 0.0f);
+    if (id / 32 < gbx::model_table_warps(n_ant, M, n_int))
+        gbx::model_table(id / 32, n_ant, M, n_fft, n_int, g0, m.tau, m.phi0, m.rate, pf, ff);
 }
 
 int fail(int code, const char* msg) {
@@ -166,9 +157,8 @@ extern "C" int corr_integrate_static(int n_ant, int n_pol, int n_fft, int n_int,
         return fail(CORR_E_CUDA, "corr_integrate_static: device query failed");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     unsigned char* base = static_cast<unsigned char*>(scratch);
-    const int64_t work = static_cast<int64_t>(n_ant) * (n_fft / 2 + n_int) + n_ant;
-    static_tables_kernel<<<static_cast<int>(std::min<int64_t>((work + 255) / 256, 4096)), 256, 0, s>>>(
-        m, n_ant, n_fft, n_int, g0, base, L);
+    const int64_t threads = std::max<int64_t>(32 * gbx::model_table_warps(n_ant, n_fft / 2, n_int), n_ant);
+    static_tables_kernel<<<static_cast<unsigned>((threads + 63) / 64), 64, 0, s>>>(m, n_ant, n_fft, n_int, g0, base, L);
     if (cudaGetLastError() != cudaSuccess ||
         gbx::launch_fengine_twiddles(n_fft, reinterpret_cast<float2*>(base + L.tw), s) != cudaSuccess)
         return fail(CORR_E_CUDA, "corr_integrate_static: table kernel");
