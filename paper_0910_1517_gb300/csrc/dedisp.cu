@@ -66,9 +66,11 @@ __device__ __forceinline__ float2 twiddle_m(int p, float inv_half_m) {
 }
 
 struct DdBlocks {
-    const float4* ring;     // [cap][n_chan] voltage spectra (X re, X im, Y re, Y im)
+    const float4* ring;     // [cap][n_chan] voltage spectra (X re, X im, Y re, Y im) of earlier pushes
+    const float4* spec;     // this push's frames, read where they are
     int64_t cap;            // frames in the ring
     int64_t start0;         // ring frame of block 0's first frame
+    int64_t old;            // unconsumed frames in the ring: frame `old` after start0 is spec's first
     int step;               // frames between blocks (F - O)
     float2* work;           // [n_blocks][F][n_chan] float4 as pairs: pol X then pol Y per element
     float* part;            // [n_blocks][n_chan / col_g(F)][keep] detected column-group sums
@@ -84,13 +86,13 @@ dd_pass_a(DdBlocks d, int n_chan, const float2* __restrict__ tw) {
     extern __shared__ float2 sm[];
     const int g = threadIdx.x / P::T, t = threadIdx.x % P::T;
     const int k0 = blockIdx.x * kColG, blk = blockIdx.y;
-    int64_t f0 = d.start0 + static_cast<int64_t>(blk) * d.step;
-    if (f0 >= d.cap) f0 -= d.cap;
+    const int64_t f0 = static_cast<int64_t>(blk) * d.step;   // from the oldest unconsumed frame
     for (int i = threadIdx.x; i < F * kColG; i += blockDim.x) {
         const int l = i / kColG, kk = i % kColG;
-        int64_t f = f0 + l;
-        if (f >= d.cap) f -= d.cap;
-        const float4 v = __ldg(d.ring + f * n_chan + k0 + kk);
+        const int64_t f = f0 + l;
+        const int64_t r = d.start0 + f;
+        const float4* row = f >= d.old ? d.spec + (f - d.old) * n_chan : d.ring + (r >= d.cap ? r - d.cap : r) * n_chan;
+        const float4 v = __ldg(row + k0 + kk);
         sm[(2 * kk) * P::PAD + pad16(l)] = make_float2(v.x, v.y);
         sm[(2 * kk + 1) * P::PAD + pad16(l)] = make_float2(v.z, v.w);
     }
@@ -413,8 +415,15 @@ int corr_dd_push_device(corr_dd_t* d, const float* spec, int64_t n_frames, float
     const size_t fb = static_cast<size_t>(d->n_chan) * sizeof(float4);
     const bool tm = d->timing && n_blocks > 0;
     if (tm) DDCU(cudaEventRecord(d->ev[0], s));
-    // append to the ring (two pieces at the wrap)
-    int64_t done = 0;
+    // The blocks read this push's frames where they are; into the ring go only those that stay
+    // unconsumed (two pieces at the wrap), behind the slots of the others.  The copy overwrites no
+    // frame that a block of this push still reads: the ring has F + max_push_frames slots.  (A
+    // copy of every frame is a read and a write that no pass needs: 554 -> 529 us for 8192 frames
+    // of 1024 channels in blocks of 4096 with 1200 overlapping.)
+    int64_t done = std::max<int64_t>(0, n_frames - (have - static_cast<int64_t>(n_blocks) * keep));
+    int64_t start0 = d->wpos - d->have;         // ring frame of the oldest unconsumed frame
+    start0 = ((start0 % d->cap) + d->cap) % d->cap;
+    d->wpos = (d->wpos + done) % d->cap;
     while (done < n_frames) {
         const int64_t take = std::min(n_frames - done, d->cap - d->wpos);
         DDCU(cudaMemcpyAsync(d->ring + d->wpos * d->n_chan, spec + done * d->n_chan * 4, take * fb,
@@ -423,9 +432,7 @@ int corr_dd_push_device(corr_dd_t* d, const float* spec, int64_t n_frames, float
         done += take;
     }
     if (n_blocks > 0) {
-        int64_t start0 = d->wpos - have;        // ring frame of the oldest unconsumed frame
-        start0 = ((start0 % d->cap) + d->cap) % d->cap;
-        DdBlocks b{d->ring, d->cap, start0, keep, d->work, d->part, keep};
+        DdBlocks b{d->ring, reinterpret_cast<const float4*>(spec), d->cap, start0, d->have, keep, d->work, d->part, keep};
         const int64_t M = static_cast<int64_t>(d->F) * d->n_chan;
         const float inv_half_m = 2.0f / static_cast<float>(M);
         const float scale = static_cast<float>(1.0 / (static_cast<double>(d->n_chan) * static_cast<double>(M)));
