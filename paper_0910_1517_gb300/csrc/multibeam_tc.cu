@@ -188,36 +188,47 @@ multibeam_tc_kernel(const float* __restrict__ spec, int n_ant, int n_pol, int n_
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_f16_f32(kRows, G.N);
-            const uint32_t lbo_a = kRows * 16, lbo_b = static_cast<uint32_t>(G.N) * 16, sbo = 128;
-            const uint32_t ah = smem_u32(a_hi), al = smem_u32(a_lo);
-            for (int st = 0; st < n_stage && !*abort_flag; ++st) {
-                const int s = st & 1;
-                if (!mbar_wait(&sh.full[s], (st >> 1) & 1, err, ERR_WAIT_STAGE) ||
-                    !mbar_wait(&sh.acce[s], ((st >> 1) & 1) ^ 1, err, ERR_WAIT_EPI)) {
-                    *abort_flag = 1;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t bh = smem_u32(b_base + static_cast<size_t>(2 * s) * G.b_bytes);
-                const uint32_t bl = bh + G.b_bytes;
-                const uint32_t d = tmem + s * 128;
-                for (int kk = 0; kk < G.KC / 2; ++kk) {
-                    const uint64_t dah = smem_desc_noswizzle(ah + kk * 2 * lbo_a, lbo_a, sbo);
-                    const uint64_t dal = smem_desc_noswizzle(al + kk * 2 * lbo_a, lbo_a, sbo);
-                    const uint64_t dbh = smem_desc_noswizzle(bh + kk * 2 * lbo_b, lbo_b, sbo);
-                    const uint64_t dbl = smem_desc_noswizzle(bl + kk * 2 * lbo_b, lbo_b, sbo);
+        // the whole warp waits and one elected lane issues: from an elect branch the products follow
+        // each other at the tensor pipe's rate (N = 128: 64 clocks; from a lane == 0 branch 129 and
+        // more).  With the converters' and drains' voted waits: 32 antennas x 2, 512 channels, 2048
+        // spectra 424 -> 414 us for 32 beams and 457 -> 439 for 64, 60 inputs and 25 beams 58 -> 50.5;
+        // the converters bound it now.
+        const uint32_t idesc = idesc_f16_f32(kRows, G.N);
+        const uint32_t lbo_a = kRows * 16, lbo_b = static_cast<uint32_t>(G.N) * 16, sbo = 128;
+        const uint32_t ah = smem_u32(a_hi), al = smem_u32(a_lo);
+        const uint64_t step_a = (2 * lbo_a) >> 4, step_b = (2 * lbo_b) >> 4;
+        const int nk = G.KC / 2;
+        for (int st = 0; st < n_stage; ++st) {
+            const int s = st & 1;
+            if (__any_sync(0xffffffffu, *abort_flag) || !mbar_wait_warp(&sh.full[s], (st >> 1) & 1, err, ERR_WAIT_STAGE) ||
+                !mbar_wait_warp(&sh.acce[s], ((st >> 1) & 1) ^ 1, err, ERR_WAIT_EPI)) {
+                *abort_flag = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t bh = smem_u32(b_base + static_cast<size_t>(2 * s) * G.b_bytes);
+            const uint32_t d = tmem + s * 128;
+            if (elect_one()) {
+                uint64_t dah = smem_desc_noswizzle(ah, lbo_a, sbo), dal = smem_desc_noswizzle(al, lbo_a, sbo);
+                uint64_t dbh = smem_desc_noswizzle(bh, lbo_b, sbo), dbl = smem_desc_noswizzle(bh + G.b_bytes, lbo_b, sbo);
+#pragma unroll 2
+                for (int kk = 0; kk < nk; ++kk) {
                     umma_f16(d, dah, dbh, idesc, kk == 0 ? 0u : 1u);
                     umma_f16(d, dah, dbl, idesc, 1u);
                     umma_f16(d, dal, dbh, idesc, 1u);
+                    dah += step_a;
+                    dal += step_a;
+                    dbh += step_b;
+                    dbl += step_b;
                 }
                 umma_commit(&sh.empty[s]);      // the B slot is free once these MMAs finish
                 umma_commit(&sh.accf[s]);       // the accumulator is complete
             }
-            umma_commit(&sh.done);
-            mbar_wait(&sh.done, 0, err, ERR_WAIT_MMA);
+            __syncwarp();
         }
+        if (elect_one()) umma_commit(&sh.done);
+        __syncwarp();
+        mbar_wait_warp(&sh.done, 0, err, ERR_WAIT_MMA);
     } else if (warp >= kConv0) {
         // ------------------------------------------------------------ converters
         const int ct = tid - kConv0 * 32;
@@ -240,13 +251,12 @@ multibeam_tc_kernel(const float* __restrict__ spec, int n_ant, int n_pol, int n_
         }
         for (int st = 0; st < n_stage; ++st) {
             const int fs = st % G.nf, s = st & 1;
-            int ok = 1;
-            if (lane == 0) {
-                ok = !*abort_flag && mbar_wait(&sh.f32full[fs], (st / G.nf) & 1, err, ERR_WAIT_STAGE) &&
-                     mbar_wait(&sh.empty[s], ((st >> 1) & 1) ^ 1, err, ERR_WAIT_MMA);
-                if (!ok) *abort_flag = 1;
+            if (__any_sync(0xffffffffu, *abort_flag) ||
+                !mbar_wait_warp(&sh.f32full[fs], (st / G.nf) & 1, err, ERR_WAIT_STAGE) ||
+                !mbar_wait_warp(&sh.empty[s], ((st >> 1) & 1) ^ 1, err, ERR_WAIT_MMA)) {
+                *abort_flag = 1;
+                break;
             }
-            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
             const float* src = reinterpret_cast<const float*>(f32_base + static_cast<size_t>(fs) * G.f32_bytes);
             unsigned char* bh = b_base + static_cast<size_t>(2 * s) * G.b_bytes;
 #pragma unroll
@@ -297,7 +307,7 @@ multibeam_tc_kernel(const float* __restrict__ spec, int n_ant, int n_pol, int n_
         float s00 = 0.f, s11 = 0.f, s01 = 0.f, sx = 0.f;
         for (int st = 0; st < n_stage; ++st) {
             const int s = st & 1;
-            if (!mbar_wait(&sh.accf[s], (st >> 1) & 1, err, ERR_WAIT_MMA)) {
+            if (!mbar_wait_warp(&sh.accf[s], (st >> 1) & 1, err, ERR_WAIT_MMA)) {
                 *abort_flag = 1;
                 break;
             }
