@@ -16,7 +16,7 @@
 //                     |y_X|^2 + |y_Y|^2 summed over the CTA's columns -> P[col group][l]
 //   D  per frame:     the column-group sums of each `avg`-sample window, scaled to a mean.
 // A and C keep two channels (four sequences: 2 x polarisation) per CTA, B one row per
-// polarisation group; every FFT runs in padded shared memory (smem_fft).
+// polarisation group; every FFT runs in padded shared memory (smem_fft, smem_fft_chain).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -45,6 +45,22 @@ std::vector<float2> smem_fft_twiddles(int L) {
     if (R3 > 1)
         for (int r = 0; r < R3; ++r)
             for (int j = 0; j < Ns3; ++j) tw.push_back(w(static_cast<double>(j) * r, static_cast<double>(L)));
+    return tw;
+}
+
+std::vector<float2> smem_fft_chain_twiddles(int L) {
+    const int R2 = (L / 16 >= 16) ? 16 : L / 16, R3 = L / (16 * R2);
+    std::vector<float2> tw = smem_fft_twiddles(L);
+    const double two_pi = 6.283185307179586476925286766559;
+    auto pass = [&](int R, int Ns) {
+        for (int r = 0; r < R; ++r)
+            for (int j = 0; j < Ns; ++j) {
+                const double ph = two_pi * (static_cast<double>(j) * r) / (static_cast<double>(R) * Ns);
+                tw.push_back(make_float2(static_cast<float>(std::cos(ph)), static_cast<float>(-std::sin(ph))));
+            }
+    };
+    if (R3 > 1) pass(R2, R3);
+    pass(16, R2 * R3);
     return tw;
 }
 
@@ -110,6 +126,8 @@ dd_pass_a(DdBlocks d, int n_chan, const float2* __restrict__ tw) {
 // B: per row k1, the frames' inverse FFTs, the twiddle, the spectrum, the chirp and the first
 // half of the inverse transform, in place.  Inverse DFTs run as conj(DFT(conj(.))), the
 // conjugations folded into the element-wise steps.  RB rows per CTA, groups g = 2 row + pol.
+// Bound by its trips through shared memory and their barriers: the points stay in registers from
+// one FFT to the next (8192 frames of 1024 channels in blocks of 4096: the push 529 -> 515 us).
 template <int NC, int RB>
 __global__ void __launch_bounds__(2 * RB * SmemFft<NC>::T, (2 * RB * SmemFft<NC>::T <= 256) ? 2 : 1)
 dd_pass_b(float2* __restrict__ work, int F, const float2* __restrict__ chirp, const float2* __restrict__ tw,
@@ -133,12 +151,14 @@ dd_pass_b(float2* __restrict__ work, int F, const float2* __restrict__ chirp, co
     float2* buf = sm + g * P::PAD;
     const float2* tr = trow + (g / 2) * NC;
     const float2* crow = crows + (g / 2) * NC;
-    // a = DFT(conj V) = conj(n_chan x~); next input n_chan x~ W^{m k1} = conj(a) W^{m k1}
-    smem_fft<NC>(buf, tw, t, g, [=](int m, float2 a) { return cmul(conjf2(a), tr[m]); });
-    // X at k2; next input conj(X C)
-    smem_fft<NC>(buf, tw, t, g, [=](int k2, float2 x) { return conjf2(cmul(x, crow[k2])); });
-    // c = DFT(conj Y) = conj(inverse DFT of Y); keep conj(c) W^{-n k1} = conj(c W^{n k1})
-    smem_fft<NC>(buf, tw, t, g, [=](int n, float2 c) { return conjf2(cmul(c, tr[n])); });
+    smem_fft_chain<NC>(
+        buf, tw, t, g,
+        // a = DFT(conj V) = conj(n_chan x~); next input n_chan x~ W^{m k1} = conj(a) W^{m k1}
+        [=](int m, float2 a) { return cmul(conjf2(a), tr[m]); },
+        // X at k2; next input conj(X C)
+        [=](int k2, float2 x) { return conjf2(cmul(x, crow[k2])); },
+        // c = DFT(conj Y) = conj(inverse DFT of Y); keep conj(c) W^{-n k1} = conj(c W^{n k1})
+        [=](int n, float2 c) { return conjf2(cmul(c, tr[n])); });
     __syncthreads();
     for (int i = threadIdx.x; i < RB * NC; i += blockDim.x) {
         const int r = i / NC, n = i % NC;
@@ -386,7 +406,7 @@ int corr_dd_create(corr_dd_t** out, int n_chan, int fft_frames, int overlap_fram
     if (cudaMalloc(&d->chirp, ch.size() * sizeof(float2)) != cudaSuccess) return bad("cudaMalloc(chirp)");
     if (cudaMemcpy(d->chirp, ch.data(), ch.size() * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
         return bad("cudaMemcpy(chirp)");
-    const std::vector<float2> twf = smem_fft_twiddles(fft_frames), twc = smem_fft_twiddles(n_chan);
+    const std::vector<float2> twf = smem_fft_twiddles(fft_frames), twc = smem_fft_chain_twiddles(n_chan);
     if (cudaMalloc(&d->tw_f, twf.size() * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&d->tw_c, twc.size() * sizeof(float2)) != cudaSuccess)
         return bad("cudaMalloc(twiddles)");
