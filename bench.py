@@ -61,7 +61,7 @@ CONFIG = {
 FORMS = {
     "fp32": "plain FP32: FP32 spectra, X-engine FP32 multiply-adds on the CUDA cores",
     "fp32tc": "FP32 spectra held as fp16 hi + lo planes (v = hi + lo to 2^-22 |v|), X-engine on tcgen05: "
-              "H H^T in 128-frame FP32 chunks, H L^T + L H^T in a separate accumulator; FP32 accuracy bound",
+              "H [H; L]^T in 512-frame FP32 chunks, L H^T as the transpose of H L^T; FP32 accuracy bound",
     "i8": "per-channel scaled int8 requantisation, exact integer X-engine on tcgen05",
     "f16": "per-channel scaled FP16 requantisation, X-engine on tcgen05 with FP32 accumulation",
     "fp32_self": "self-polar (total-intensity) mode of the plain FP32 form: products RR*, LL* only "
@@ -512,7 +512,13 @@ def run_dedisp_leg(corr, torch, pk, k=20, dm=30.0, f_lo=1780.0 / 3.0, bw=100.0 /
         st = [float(x) / max(cnt, 1) for x in st]
         nb = n_out / k / keep                               # blocks per push, averaged (one output per frame)
         M = F * N_CHAN
-        traffic = {"ring_copy": 2 * n_push * N_CHAN * 16, "A": nb * 2 * M * 16, "B": nb * (2 * M * 16 + M * 8),
+        # into the ring go the frames of a push that stay unconsumed (averaged over many pushes)
+        have = copied = 0
+        for _ in range(keep):
+            have += n_push
+            have -= max(0, (have - F) // keep + 1) * keep
+            copied += min(n_push, have)
+        traffic = {"ring_copy": 2 * copied / keep * N_CHAN * 16, "A": nb * 2 * M * 16, "B": nb * (2 * M * 16 + M * 8),
                    "C": nb * (M * 16 + keep * (N_CHAN // 2) * 4), "D": nb * keep * (N_CHAN // 2) * 4}
         traffic = {q: int(b) for q, b in traffic.items()}
         names = ["ring_copy", "A", "B", "C", "D"]

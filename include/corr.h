@@ -29,7 +29,8 @@
  * (e = log2(n_fft) - 8, so |v| < 2^15 for any int8 input) is stored as fp16
  * hi = rn(v), lo = rn(v - hi), which holds v to 2^-22 |v|; the Gram is
  * H H^T + H L^T + L H^T with exact fp16 products, accumulated in FP32 over
- * 128-frame chunks that are added in FP32, then multiplied by 2^2e.  No scales
+ * chunks (512 frames for 64 inputs, 128 otherwise) that are added in FP32,
+ * then multiplied by 2^2e.  No scales
  * are needed.  Beams are always formed from the FP32 spectra.
  *
  * Ownership: the library allocates and owns every device buffer and one CUDA
