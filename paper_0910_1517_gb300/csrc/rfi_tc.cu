@@ -26,7 +26,8 @@
 //
 // What bounds it: an MMA with N = 16 or 32 takes the tensor core about 40 cycles whatever its N, 144
 // of them a strip (0.6 ms for 4096 patches), and the near ties' sums, one after another by
-// definition, which little runs beside.  4096 patches: 1.65 ms; 10.95 ms with a CUDA-core kernel a
+// definition, which little runs beside.  4096 patches, four launches: 1.64 ms (1.82 with the near
+// ties' operands converted to FP32 first); 10.95 ms with a CUDA-core kernel a
 // layer and the head's (conv2 5.0, conv3 5.5, conv1 0.29, head 0.15 ms).  Layer 1's four positions a
 // thread: with one, its weight loads took the pass to 1.97 ms.
 #include <type_traits>
@@ -88,6 +89,13 @@ __device__ __forceinline__ uint32_t round_pair(uint32_t v0, uint32_t v1, float b
     return *reinterpret_cast<const uint32_t*>(&a);
 }
 
+// w a + acc in FP32, rounded once, w and a fp16: the same value as of the operands converted first, in
+// one instruction instead of three (flagging 4096 patches 2.05 -> 1.87 ms)
+__device__ __forceinline__ float fma_half(unsigned short w, unsigned short a, float acc) {
+    asm("fma.rn.f32.f16 %0, %1, %2, %0;" : "+f"(acc) : "h"(w), "h"(a));
+    return acc;
+}
+
 // The activation of output channel o at plane index `at` (the tap (0, 0) of its position), summed in
 // FP32 in the order of the CUDA-core kernels: bias, then channel by channel, tap by tap.  GROUPS
 // planes of 8 channels of `pos` positions; wt: packed weights of (o, channel 0, tap 0), `wg` bytes
@@ -109,9 +117,7 @@ __device__ __forceinline__ __half sum_in_order(const unsigned char* planes, int 
 #pragma unroll
             for (int tap = 0; tap < 9; ++tap) {
                 const uint32_t aw = (&a[tap].x)[ch / 2], ww = (&w[tap].x)[ch / 2];
-                const float2 af = __half22float2(*reinterpret_cast<const __half2*>(&aw));
-                const float2 wf = __half22float2(*reinterpret_cast<const __half2*>(&ww));
-                acc = (ch & 1) ? fmaf(wf.y, af.y, acc) : fmaf(wf.x, af.x, acc);
+                acc = fma_half(static_cast<unsigned short>(ww >> (16 * (ch & 1))), static_cast<unsigned short>(aw >> (16 * (ch & 1))), acc);
             }
     }
     return __float2half_rn(fmaxf(acc, 0.0f));
