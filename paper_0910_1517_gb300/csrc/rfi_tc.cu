@@ -14,11 +14,15 @@
 //
 // Rounding.  The tensor core adds the products of an output in another order than the CUDA-core
 // kernels; where the FP32 sum lies next to a rounding boundary of fp16 the activation could round
-// the other way, a whole fp16 step.  Activations of layers 2 and 3 within 64 FP32 steps of a boundary
-// (1.6 % of them) are therefore listed and summed again in FP32 in the CUDA-core order, one a
-// thread: on 4096 patches the probabilities are then within 5e-7 to 9e-7 (relative 2-norm) of that
-// order's and 4e-4 at most; within 16 steps 2.5e-6 and 7.5e-4, 0.2 ms less; with none 1.6e-5 and up
-// to 2.9e-3, 0.7 ms less of the 1.65 ms.
+// the other way, a whole fp16 step.  Activations near a boundary are therefore listed and summed
+// again in FP32 in the CUDA-core order, one a thread.  How near is set by what the sums' errors follow:
+// in layer 2, whose flips spread over nine positions and sixteen channels, the size of the terms
+// (kTie2 x the mean of the output's |weights| x the sum of its 144 inputs; small sums of large
+// terms are the ones that flip furthest from a boundary), in layer 3 32 FP32 steps of the sum.
+// Largest differences of the probabilities from the CUDA-core order's, 40 x 4096 patches with as many
+// networks: 3e-4 (median of the 40), 6.6e-4 (worst), relative 2-norm at most 6e-7; the same with
+// twice and six times the margin.  With 64 steps of the sum in both layers, as fast within 10 %, 6e-4 and
+// 1.2e-3; with 256, a third slower, 4e-4 and 8.7e-4.
 //
 // Roles: warp 8 issues the MMAs of a layer tile by tile (a commit each), warps 0-7 take the tiles as
 // they complete: bias, ReLU, rounding to fp16, zeros outside the image, and the next layer's
@@ -26,8 +30,7 @@
 //
 // What bounds it: an MMA with N = 16 or 32 takes the tensor core about 40 cycles whatever its N, 144
 // of them a strip (0.6 ms for 4096 patches), and the near ties' sums, one after another by
-// definition, which little runs beside.  4096 patches, four launches: 1.64 ms (1.82 with the near
-// ties' operands converted to FP32 first); 10.95 ms with a CUDA-core kernel a
+// definition, which little runs beside.  4096 patches, four launches: 1.8 ms; 10.95 ms with a CUDA-core kernel a
 // layer and the head's (conv2 5.0, conv3 5.5, conv1 0.29, head 0.15 ms).  Layer 1's four positions a
 // thread: with one, its weight loads took the pass to 1.97 ms.
 #include <type_traits>
@@ -58,7 +61,8 @@ struct Smem {
     static constexpr int A2 = A1 + 2 * kPos1 * 16;                           // 4 planes
     static constexpr int x = A2 + 4 * kPos2 * 16;                            // 14 input rows, FP32
     static constexpr int ties = x + 14 * kXPitch * 4;                        // list of near ties (position * 32 + channel)
-    static constexpr int total = ties + kMaxTies * 2;
+    static constexpr int sum1 = ties + kMaxTies * 2;                         // layer 1's activations summed over channels, FP32
+    static constexpr int total = sum1 + kPos1 * 4;
 };
 static_assert(8 * kPosA3 * 4 <= 2 * kPos1 * 16 && kTiles2 * 128 * 32 <= 65536, "A3 where A1 was; 16-bit list entries");
 static_assert(Smem::total <= 112 * 1024, "two CTAs an SM");
@@ -70,22 +74,34 @@ struct alignas(16) Ctl {
     int fail, n_tie[2];                                   // near ties of layers 2 and 3
     float bias[16 + 32 + 16 + 16 + 1];                    // b1, b2, b3, w4, b4
     float4 w1[2][9][2];                                   // layer 1, [8 channels][tap][4 channels]
+    float tie2[32];                                       // layer 2: kTie2 x the mean of an output's |weights|
 };
 
-// r >= 0 within kTieBand FP32 steps of the middle between two fp16 numbers, where rounding turns:
-// the 13 bits that fp16 drops lie around 0x1000 (below fp16's normal numbers and above its largest
-// the answer does not matter)
-constexpr uint32_t kTieBand = 64;
-__device__ __forceinline__ bool near_tie(float r) {
-    return ((__float_as_uint(r) - (0x1000u - kTieBand)) & 0x1fffu) <= 2 * kTieBand;
+// Near ties of layer 2: r > 0 within e of the middle between two fp16 numbers, where rounding turns;
+// kTie2Cap r, a quarter to half of the way between the two, is the most it reaches (small sums of
+// large terms would all be listed, and their flips weigh little).
+constexpr float kTie2 = 8.0f / 16777216.0f, kTie2Cap = 1.0f / 8192.0f;
+__device__ __forceinline__ bool near_tie2(float r, float e) {
+    const float mid = __uint_as_float((__float_as_uint(r) & ~0x1fffu) | 0x1000u);
+    return fabsf(r - mid) < fminf(e, r * kTie2Cap);
 }
 
-// A pair of activations (channels o and o + 1) from their sums without bias; their near ties in mask
-__device__ __forceinline__ uint32_t round_pair(uint32_t v0, uint32_t v1, float b0, float b1, int o, uint32_t& mask) {
+// ... of layer 3: r >= 0 within kTie3 FP32 steps of it: the 13 bits that fp16 drops lie around 0x1000
+// (below fp16's normal numbers and above its largest the answer does not matter)
+constexpr uint32_t kTie3 = 32;
+__device__ __forceinline__ bool near_tie3(float r) {
+    return ((__float_as_uint(r) - (0x1000u - kTie3)) & 0x1fffu) <= 2 * kTie3;
+}
+
+// A pair of activations (channels o and o + 1) from their sums without bias; their near ties, as the
+// functions t0 and t1 find them, in mask
+template <typename T0, typename T1>
+__device__ __forceinline__ uint32_t round_pair(uint32_t v0, uint32_t v1, float b0, float b1, int o, uint32_t& mask, const T0& t0,
+                                               const T1& t1) {
     const float r0 = fmaxf(__uint_as_float(v0) + b0, 0.0f), r1 = fmaxf(__uint_as_float(v1) + b1, 0.0f);
     const __half2 a = __floats2half2_rn(r0, r1);
-    if (near_tie(r0)) mask |= 1u << o;
-    if (near_tie(r1)) mask |= 2u << o;
+    if (t0(r0)) mask |= 1u << o;
+    if (t1(r1)) mask |= 2u << o;
     return *reinterpret_cast<const uint32_t*>(&a);
 }
 
@@ -153,7 +169,14 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
     const uint32_t tm = __shfl_sync(0xffffffffu, c.taddr, 0);
     const uint32_t s0 = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
     float* xs = reinterpret_cast<float*>(smem + Smem::x);
+    float* sum1 = reinterpret_cast<float*>(smem + Smem::sum1);
     bool ok = mbar_wait_warp(&c.wbar, 0, p.err, ERR_WAIT_STAGE);
+    if (tid < 32) {
+        float m = 0.0f;
+        for (int q = 0; q < 144; ++q)
+            m += fabsf(__half2float(*reinterpret_cast<const __half*>(smem + Smem::pack + rfi_pack2(tid, q / 9, q % 9))));
+        c.tie2[tid] = m * (kTie2 / 144.0f);
+    }
 
     // this thread's 16 bytes of the strip's 14 input rows (y0 - 3 .. y0 + 10), zero outside the patch
     const int n_items = p.B * kStrips;
@@ -229,6 +252,7 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
                 in[j] = cc > 0 && q < kRows1 * kPitch && gy >= 0 && gy < kPatch;
                 at[j] = in[j] ? r * kXPitch + cc - 1 : 0;
             }
+            float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
             for (int g = 0; g < 2; ++g) {
                 float2 acc[4][4];
@@ -255,12 +279,15 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
                     uint32_t h[4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const __half2 a = __floats2half2_rn(fmaxf(acc[j][e].x, 0.0f), fmaxf(acc[j][e].y, 0.0f));
+                        const float ax = fmaxf(acc[j][e].x, 0.0f), ay = fmaxf(acc[j][e].y, 0.0f);
+                        const __half2 a = __floats2half2_rn(ax, ay);
                         h[e] = in[j] ? *reinterpret_cast<const uint32_t*>(&a) : 0u;
+                        sum[j] += ax + ay;
                     }
                     if (q <= kRows1 * kPitch)              // (the position after the last row: its right edge)
                         reinterpret_cast<uint4*>(smem + Smem::A1)[g * kPos1 + q + 1] = make_uint4(h[0], h[1], h[2], h[3]);
                     const int r = q / kPitch;
+                    if (g && q <= kRows1 * kPitch) sum1[q + 1] = in[j] ? sum[j] : 0.0f;
                     if (KEEP && in[j] && r >= 2 && r < 10) keep(p.A1 + g * 8 * kPatch * kPatch, 16, 8, h, patch, y0 - 2 + r, q % kPitch - 1);
                 }
             }
@@ -281,10 +308,16 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
                 tmem_wait_ld();
                 const int q = t * 128 + 32 * q4 + lane, r = q / kPitch, cc = q % kPitch, gy = y0 - 1 + r;
                 const bool in = cc > 0 && r < 10 && gy >= 0 && gy < kPatch;
+                float near = 0.0f;                         // the inputs' sum over channels and taps
+#pragma unroll
+                for (int tap = 0; tap < 9; ++tap) near += sum1[q + (tap / 3) * kPitch + tap % 3];
                 uint32_t h[16], mask = 0;
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
-                    h[e] = round_pair(v[2 * e], v[2 * e + 1], c.bias[16 + 2 * e], c.bias[17 + 2 * e], 2 * e, mask);
+                    h[e] = round_pair(
+                        v[2 * e], v[2 * e + 1], c.bias[16 + 2 * e], c.bias[17 + 2 * e], 2 * e, mask,
+                        [&](float r) { return near_tie2(r, near * c.tie2[2 * e]); },
+                        [&](float r) { return near_tie2(r, near * c.tie2[2 * e + 1]); });
                     if (!in) h[e] = 0u;
                 }
                 uint4* d = reinterpret_cast<uint4*>(smem + Smem::A2) + q + 1;
@@ -330,7 +363,8 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
                 uint32_t mask = 0;
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
-                    a3[e * kPosA3 + q] = round_pair(v[2 * e], v[2 * e + 1], c.bias[48 + 2 * e], c.bias[49 + 2 * e], 2 * e, mask);
+                    a3[e * kPosA3 + q] =
+                        round_pair(v[2 * e], v[2 * e + 1], c.bias[48 + 2 * e], c.bias[49 + 2 * e], 2 * e, mask, near_tie3, near_tie3);
                 list(cc > 0 && r < kRows ? mask : 0u, q, 1);
             }
             tc_fence_before();
