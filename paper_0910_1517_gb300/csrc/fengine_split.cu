@@ -8,8 +8,10 @@ namespace gbx {
 namespace {
 
 // The beams of the shared frame blocks, parts added in order: sum of the incoherent sums, and per
-// polarisation the detected sum of the voltage sums.  Four channels a thread.
-__global__ void beam_combine_kernel(const FeSplit sp, int n_pol, int n_chan, int first, int n_int, float* __restrict__ beams) {
+// polarisation the detected sum of the voltage sums.  Four channels a thread, stored together where
+// `wide`: the beams can be a caller's (corr_integrate_static), at any address of a float.
+__global__ void beam_combine_kernel(const FeSplit sp, int n_pol, int n_chan, int first, int n_int, bool wide,
+                                    float* __restrict__ beams) {
     const int64_t n = static_cast<int64_t>(sp.frames) * n_chan;
     for (int64_t q = 4 * (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x); q < n;
          q += 4 * static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -31,8 +33,15 @@ __global__ void beam_combine_kernel(const FeSplit sp, int n_pol, int n_chan, int
             for (int e = 0; e < 4; ++e) pw[e] += fmaf(c[e].y, c[e].y, c[e].x * c[e].x);
         }
         float* b = beams + static_cast<int64_t>(first) * n_chan + q;
-        *reinterpret_cast<float4*>(b) = inc;
-        *reinterpret_cast<float4*>(b + static_cast<int64_t>(n_int) * n_chan) = make_float4(pw[0], pw[1], pw[2], pw[3]);
+        float* bc = b + static_cast<int64_t>(n_int) * n_chan;
+        if (wide) {
+            *reinterpret_cast<float4*>(b) = inc;
+            *reinterpret_cast<float4*>(bc) = make_float4(pw[0], pw[1], pw[2], pw[3]);
+        } else {
+            b[0] = inc.x, b[1] = inc.y, b[2] = inc.z, b[3] = inc.w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) bc[e] = pw[e];
+        }
     }
 }
 
@@ -84,8 +93,10 @@ cudaError_t launch_fengine_split(const FeParams& p, int mode, const FeSplit& sp,
     }
     if (e != cudaSuccess) return e;
     const int64_t quads = static_cast<int64_t>(sp.frames) * p.n_chan / 4;
+    // every row of n_chan floats lies as the first one does
+    const bool wide = (reinterpret_cast<uintptr_t>(p.beams) & 15) == 0;
     beam_combine_kernel<<<static_cast<int>(std::min<int64_t>((quads + 255) / 256, 4096)), 256, 0, s>>>(
-        sp, p.n_pol, p.n_chan, p.n_int - sp.frames, p.n_int, p.beams);
+        sp, p.n_pol, p.n_chan, p.n_int - sp.frames, p.n_int, wide, p.beams);
     return cudaGetLastError();
 }
 
