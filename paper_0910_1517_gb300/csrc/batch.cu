@@ -25,6 +25,20 @@
 
 using namespace gbx;
 
+// What a branch's nodes are captured with beside the F-engine's parameters: buffers and settings that
+// corr_set_power_dump and corr_set_mode change on a handle while it belongs to a batch.
+struct Captured {
+    const float* dump_part = nullptr;
+    float* power = nullptr;
+    const float* beams_raw = nullptr;
+    float* beams = nullptr;
+    int dump = 0, beam_avg = 0, polmode = 0;
+    bool operator==(const Captured& o) const {
+        return dump_part == o.dump_part && power == o.power && beams_raw == o.beams_raw && beams == o.beams && dump == o.dump &&
+               beam_avg == o.beam_avg && polmode == o.polmode;
+    }
+};
+
 struct corr_batch {
     int n_sub = 0;
     corr* h[kMaxSub] = {};
@@ -38,7 +52,7 @@ struct corr_batch {
     int64_t* d_g0 = nullptr;
     FeParams fe_p[kMaxSub] = {};              // F-engine parameters of the next replay
     FeParams cap_p[kMaxSub] = {};             // ... and those the graph was captured with
-    int cap_dump[kMaxSub] = {};
+    Captured cap_s[kMaxSub];
     cudaGraphNode_t fe_node[kMaxSub] = {};    // the F-engine kernel node of each branch
     cudaKernelNodeParams fe_kp[kMaxSub] = {};
     XtBatch* h_xt = nullptr;     // pinned, one one-entry table per sub-array
@@ -109,6 +123,18 @@ FeParams fe_params(corr* h, const int8_t* x, int64_t ld, int64_t n_avail) {
     fp.tw = h->d_tw;
     fp.err = h->d_err;
     return fp;
+}
+
+Captured captured_of(const corr* h) {
+    Captured c;
+    c.dump_part = h->d_dump_part;
+    c.power = h->d_power;
+    c.beams_raw = h->d_beams_raw;
+    c.beams = h->d_beams;
+    c.dump = h->dump;
+    c.beam_avg = h->beam_avg;
+    c.polmode = h->polmode;
+    return c;
 }
 
 // Branch q of the graph: sub-array q's whole integration on stream s.
@@ -187,7 +213,7 @@ int capture(corr_batch* b) {
     BCU(cudaGraphInstantiate(&b->exec, g, 0));
     for (int q = 0; q < b->n_sub; ++q) {
         b->cap_p[q] = b->fe_p[q];
-        b->cap_dump[q] = b->h[q]->dump;
+        b->cap_s[q] = captured_of(b->h[q]);
     }
     for (int q = 0; q < b->n_sub; ++q) BCU(cudaGraphKernelNodeGetParams(b->fe_node[q], &b->fe_kp[q]));
     return CORR_OK;
@@ -306,8 +332,8 @@ int corr_batch_integrate_device(corr_batch_t* b, const int8_t* const* x, const i
     for (int q = 0; q < b->n_sub; ++q)
         if (fengine_clustered(b->h[q]->n_chan, b->fmode[q]) && std::memcmp(&b->fe_p[q], &b->cap_p[q], sizeof(FeParams)))
             recapture = true;
-    for (int q = 0; q < b->n_sub; ++q)   // the dumps' buffers are the capture's
-        if (b->fe_p[q].dump != b->cap_p[q].dump || b->h[q]->dump != b->cap_dump[q]) recapture = true;
+    for (int q = 0; q < b->n_sub; ++q)
+        if (!(captured_of(b->h[q]) == b->cap_s[q])) recapture = true;
     if (recapture)
         if (int rc = capture(b)) return rc;
     for (int q = 0; q < b->n_sub; ++q) {   // this integration's sample pointers into the F-engine nodes
