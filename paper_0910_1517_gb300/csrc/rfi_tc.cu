@@ -51,7 +51,9 @@ static_assert(kTiles2 * 128 + 2 * kPitch + 2 <= kPos1 && kTiles3 * 128 + 2 * kPi
 constexpr int kEpiWarps = 8;
 constexpr int kThreadsTc = (kEpiWarps + 1) * 32;
 
-// near ties a layer of a strip can list; more (patches of one repeated value) stay as they are
+// near ties a layer of a strip can list.  With more of them (patches of one repeated value: a channel's
+// positions are all near ties or none) the whole layer of the strip is summed in order instead: which
+// of them found a place on the list would depend on the warps' timing.
 constexpr int kMaxTies = 2048;
 constexpr int kPosA3 = kTiles3 * 128;                     // A3 [8 channel pairs][position], where A1 was
 
@@ -160,7 +162,8 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
     if (tid < 144) reinterpret_cast<float*>(c.w1)[((tid / 72) * 9 + tid % 9) * 8 + (tid / 9) % 8] = __half2float(p.w1[tid]);
     for (int q = tid; q < 81; q += kThreadsTc)
         c.bias[q] = __half2float(q < 16 ? p.b1[q] : q < 48 ? p.b2[q - 16] : q < 64 ? p.b3[q - 48] : q < 80 ? p.w4[q - 64] : p.b4[0]);
-    // zero everything once: guard positions before and after the planes stay zero (finite) for good
+    // zero everything once: the guard positions before and after the planes.  (A3 overwrites A1's; only
+    // positions outside the strip read them, whose sums are not used.)
     for (int q = tid; q < (Smem::total - Smem::A1) / 16; q += kThreadsTc)
         reinterpret_cast<uint4*>(smem + Smem::A1)[q] = make_uint4(0u, 0u, 0u, 0u);
     tc_fence_before();
@@ -328,8 +331,16 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
             tc_fence_before();
         }
         __syncthreads();
-        for (int i = tid; i < min(c.n_tie[0], kMaxTies); i += kThreadsTc) {
-            const int q = ties[i] >> 5, o = ties[i] & 31;
+        const int ties2 = c.n_tie[0];
+        for (int i = tid; i < (ties2 > kMaxTies ? 10 * kPatch * 32 : ties2); i += kThreadsTc) {
+            int q, o;
+            if (ties2 <= kMaxTies) {
+                q = ties[i] >> 5, o = ties[i] & 31;
+            } else {                                       // every position inside the image, channel by channel
+                const int r = (i / kPatch) % 10;
+                if (y0 - 1 + r < 0 || y0 - 1 + r >= kPatch) continue;
+                q = r * kPitch + i % kPatch + 1, o = i / (10 * kPatch);
+            }
             reinterpret_cast<__half*>(smem + Smem::A2)[((o / 8) * kPos2 + q + 1) * 8 + o % 8] =
                 sum_in_order<2>(smem + Smem::A1, kPos1, q, smem + Smem::pack + rfi_pack2(o, 0, 0), 512, c.bias[16 + o]);
         }
@@ -371,8 +382,11 @@ __global__ void __launch_bounds__(kThreadsTc, 2) rfi_forward_kernel(const RfiFwd
             if (!ok) *(volatile int*)&c.fail = 1;
         }
         __syncthreads();
-        for (int i = tid; i < min(c.n_tie[1], kMaxTies); i += kThreadsTc) {
-            const int q = ties[i] >> 5, o = ties[i] & 31;
+        const int ties3 = c.n_tie[1];
+        for (int i = tid; i < (ties3 > kMaxTies ? kRows * kPatch * 16 : ties3); i += kThreadsTc) {
+            const bool all = ties3 > kMaxTies;
+            const int q = all ? (i / kPatch) % kRows * kPitch + i % kPatch + 1 : ties[i] >> 5;
+            const int o = all ? i / (kRows * kPatch) : ties[i] & 31;
             reinterpret_cast<__half*>(a3)[((o / 2) * kPosA3 + q) * 2 + (o & 1)] =
                 sum_in_order<4>(smem + Smem::A2, kPos2, q, smem + Smem::pack + rfi_pack3(o, 0, 0), 256, c.bias[48 + o]);
         }
