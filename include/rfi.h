@@ -21,6 +21,13 @@
  * column = channel), masks and flags uint8 [B][64][64], probabilities float
  * [B][64][64].  Return codes are those of corr.h (CORR_OK = 0, CORR_E_*);
  * corr_last_error() describes a failure.
+ *
+ * The waits inside the FP16 flagger's forward pass are bounded.  One that runs out (a hardware or
+ * driver failure: none is expected) is recorded in a sticky error word of the network, and the
+ * calls that only queue work, rfi_infer and rfi_train_step without loss, return before it can be
+ * seen.  rfi_status, rfi_get_params, rfi_loss_grad and rfi_train_step with loss report it as
+ * CORR_E_TIMEOUT, once, and clear it: results queued since the last of these calls are then invalid.
+ * While the word is set no Adam step is taken; the weights stay as they were.
  */
 #ifndef GB300_RFI_H
 #define GB300_RFI_H
@@ -63,8 +70,16 @@ int rfi_loss_grad(rfi_net_t* net, const uint16_t* x, const uint8_t* mask, int B,
 int rfi_train_step(rfi_net_t* net, const uint16_t* x, const uint8_t* mask, int B, float lr, float* loss,
                    void* stream);
 
-/* Flag probabilities sigmoid(logit) for a batch (device out [B][64][64]). */
+/* Flag probabilities sigmoid(logit) for a batch (device out [B][64][64]), queued on stream. */
 int rfi_infer(rfi_net_t* net, const uint16_t* x, int B, float* prob, void* stream);
+
+/* Wait for stream; CORR_E_TIMEOUT if a wait of the calls queued on the network ran out (see above). */
+int rfi_status(rfi_net_t* net, void* stream);
+
+/* Failure detection without a fault: record a wait that nothing completes (about two seconds, the
+ * budget of every bounded wait) in the network's error word, as corr_wait_selftest does for itself.
+ * Synchronous; returns CORR_OK when the wait gave up and was recorded. */
+int rfi_wait_selftest(rfi_net_t* net);
 
 /* Cut power dumps P [n_in][n_dump][n_chan] (device, float) into 64 x 64 patches
  * b = (i * (n_dump/64) + d/64) * (n_chan/64) + k/64 and, per patch, compute the

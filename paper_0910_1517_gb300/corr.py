@@ -80,6 +80,8 @@ SIGNATURES = {
     "rfi_loss_grad": ([_P, _P, _P, _I, ctypes.POINTER(ctypes.c_float), _P, _P], _I),
     "rfi_train_step": ([_P, _P, _P, _I, ctypes.c_float, ctypes.POINTER(ctypes.c_float), _P], _I),
     "rfi_infer": ([_P, _P, _I, _P, _P], _I),
+    "rfi_status": ([_P, _P], _I),
+    "rfi_wait_selftest": ([_P], _I),
     "rfi_patches": ([_P, _I, _I, _I, ctypes.c_float, _P, _P, _P, _P], _I),
 }
 
@@ -415,6 +417,16 @@ def rfi_train_step(net, x, mask, B: int, lr: float, want_loss: bool = False, str
 
 def rfi_infer(net, x, B: int, prob, stream=None):
     return _ok(load().rfi_infer(net, _ptr(x), B, _ptr(prob), _stream(stream)))
+
+
+def rfi_status(net, stream=None):
+    """Wait for the stream; CorrError (CORR_E_TIMEOUT) if a bounded wait of the network's queued calls ran out."""
+    return _ok(load().rfi_status(net, _stream(stream)))
+
+
+def rfi_wait_selftest(net):
+    """Record a wait that nothing completes in the network's error word (about two seconds)."""
+    return _ok(load().rfi_wait_selftest(net))
 
 
 def rfi_patches(power, n_in: int, n_dump: int, n_chan: int, M: float, x=None, flags=None, stats=None, stream=None):

@@ -87,6 +87,10 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, u
     return true;
 }
 
+// One wait that nothing completes, recorded in *err as ERR_WAIT_STAGE once its budget is spent
+// (selftest.cu); *cycles, if given, receives how long that took.
+cudaError_t launch_wait_selftest(unsigned* err, long long* cycles, cudaStream_t s);
+
 // 1-D bulk copy global -> shared through the TMA engine, completing on `bar`.
 // dst, src 16-byte aligned; bytes a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {

@@ -366,8 +366,10 @@ __global__ void transform_kernel(const float* __restrict__ p, Wts<TA> w) {
     }
 }
 
+// err: the network's error word; gradients of a forward pass whose wait ran out are not applied
 __global__ void adam_kernel(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, float lr, float b1t, float b2t) {
+                            const float* __restrict__ g, float lr, float b1t, float b2t, const unsigned* __restrict__ err) {
+    if (*err) return;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < NPAR; q += gridDim.x * blockDim.x) {
         const float gq = g[q];
@@ -762,7 +764,7 @@ int rfi_train_step(rfi_net_t* n, const uint16_t* x, const uint8_t* mask, int B, 
     if (int rc = forward_backward(n, x, mask, B, s)) return rc;
     n->step += 1;
     const float b1t = std::pow(0.9f, static_cast<float>(n->step)), b2t = std::pow(0.999f, static_cast<float>(n->step));
-    adam_kernel<<<(NPAR + 255) / 256, 256, 0, s>>>(n->p, n->m, n->v, n->g, lr, b1t, b2t);
+    adam_kernel<<<(NPAR + 255) / 256, 256, 0, s>>>(n->p, n->m, n->v, n->g, lr, b1t, b2t, n->err);
     RCU(cudaGetLastError());
     if (int rc = transform(n, s)) return rc;
     if (loss) {
@@ -781,6 +783,21 @@ int rfi_infer(rfi_net_t* n, const uint16_t* x, int B, float* prob, void* stream)
     if (!n->fp32 && !(reinterpret_cast<uintptr_t>(x) & 15)) return forward_tc(n, x, B, prob, false, s);
     if (int rc = n->fp32 ? forward_t<float>(n, x, B, s) : forward_t<__half>(n, x, B, s)) return rc;
     return head_infer(n, B, prob, s);
+}
+
+int rfi_status(rfi_net_t* n, void* stream) {
+    if (!n) return rfail(CORR_E_INVAL, "null network");
+    RCU(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
+    return check_err(n);
+}
+
+int rfi_wait_selftest(rfi_net_t* n) {
+    if (!n) return rfail(CORR_E_INVAL, "null network");
+    RCU(gbx::launch_wait_selftest(n->err, nullptr, nullptr));
+    RCU(cudaDeviceSynchronize());
+    unsigned err = 0;
+    RCU(cudaMemcpy(&err, n->err, sizeof err, cudaMemcpyDeviceToHost));
+    return (err & gbx::ERR_WAIT_STAGE) ? CORR_OK : rfail(CORR_E_STATE, "the wait did not give up");
 }
 
 int rfi_patches(const float* power, int n_in, int n_dump, int n_chan, float M, uint16_t* x, uint8_t* mad_flags,

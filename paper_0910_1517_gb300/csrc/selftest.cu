@@ -25,12 +25,18 @@ __global__ void wait_selftest_kernel(unsigned* err, long long* cycles) {
     if (threadIdx.x == 0) {
         const long long t0 = clock64();
         const bool ok = mbar_wait(&bar, 0, err, ERR_WAIT_STAGE);   // phase 0 needs two arrivals: none come
-        *cycles = clock64() - t0;
+        if (cycles) *cycles = clock64() - t0;
         if (ok) atomicOr(err, kCompleted);
     }
 }
 
 }  // namespace
+
+cudaError_t launch_wait_selftest(unsigned* err, long long* cycles, cudaStream_t s) {
+    wait_selftest_kernel<<<1, 32, 0, s>>>(err, cycles);
+    return cudaGetLastError();
+}
+
 }  // namespace gbx
 
 using namespace gbx;
@@ -46,10 +52,7 @@ extern "C" int corr_wait_selftest(long long* cycles_out) {
     unsigned err = 0;
     long long cyc = 0;
     cudaError_t e = cudaMemset(d_err, 0, sizeof(unsigned));
-    if (e == cudaSuccess) {
-        wait_selftest_kernel<<<1, 32>>>(d_err, d_cyc);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = launch_wait_selftest(d_err, d_cyc, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpy(&err, d_err, sizeof err, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(&cyc, d_cyc, sizeof cyc, cudaMemcpyDeviceToHost);
