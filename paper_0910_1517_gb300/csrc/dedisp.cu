@@ -48,22 +48,6 @@ std::vector<float2> smem_fft_twiddles(int L) {
     return tw;
 }
 
-std::vector<float2> smem_fft_chain_twiddles(int L) {
-    const int R2 = (L / 16 >= 16) ? 16 : L / 16, R3 = L / (16 * R2);
-    std::vector<float2> tw = smem_fft_twiddles(L);
-    const double two_pi = 6.283185307179586476925286766559;
-    auto pass = [&](int R, int Ns) {
-        for (int r = 0; r < R; ++r)
-            for (int j = 0; j < Ns; ++j) {
-                const double ph = two_pi * (static_cast<double>(j) * r) / (static_cast<double>(R) * Ns);
-                tw.push_back(make_float2(static_cast<float>(std::cos(ph)), static_cast<float>(-std::sin(ph))));
-            }
-    };
-    if (R3 > 1) pass(R2, R3);
-    pass(16, R2 * R3);
-    return tw;
-}
-
 namespace {
 
 constexpr double kDispConst = 4.148808e3;   // s MHz^2 pc^-1 cm^3: delay = D DM / nu^2
@@ -127,7 +111,7 @@ dd_pass_a(DdBlocks d, int n_chan, const float2* __restrict__ tw) {
 // half of the inverse transform, in place.  Inverse DFTs run as conj(DFT(conj(.))), the
 // conjugations folded into the element-wise steps.  RB rows per CTA, groups g = 2 row + pol.
 // Bound by its trips through shared memory and their barriers: the points stay in registers from
-// one FFT to the next (8192 frames of 1024 channels in blocks of 4096: the push 529 -> 515 us).
+// one FFT to the next (8192 frames of 1024 channels in blocks of 4096: the push 529 -> 512 us).
 template <int NC, int RB>
 __global__ void __launch_bounds__(2 * RB * SmemFft<NC>::T, (2 * RB * SmemFft<NC>::T <= 256) ? 2 : 1)
 dd_pass_b(float2* __restrict__ work, int F, const float2* __restrict__ chirp, const float2* __restrict__ tw,
@@ -406,7 +390,7 @@ int corr_dd_create(corr_dd_t** out, int n_chan, int fft_frames, int overlap_fram
     if (cudaMalloc(&d->chirp, ch.size() * sizeof(float2)) != cudaSuccess) return bad("cudaMalloc(chirp)");
     if (cudaMemcpy(d->chirp, ch.data(), ch.size() * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
         return bad("cudaMemcpy(chirp)");
-    const std::vector<float2> twf = smem_fft_twiddles(fft_frames), twc = smem_fft_chain_twiddles(n_chan);
+    const std::vector<float2> twf = smem_fft_twiddles(fft_frames), twc = smem_fft_twiddles(n_chan);
     if (cudaMalloc(&d->tw_f, twf.size() * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&d->tw_c, twc.size() * sizeof(float2)) != cudaSuccess)
         return bad("cudaMalloc(twiddles)");

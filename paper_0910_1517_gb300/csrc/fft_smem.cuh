@@ -187,64 +187,51 @@ __device__ __forceinline__ void smem_fft(float2* buf, const float2* __restrict__
 
 // Three forward FFTs of the same points one after the other, output i of the first two going
 // through post1 / post2 into input i of the next, the last one's stored as post3.  A last pass of
-// radix R leaves a thread the points b + r L/R that a first pass of radix R takes, so the second
-// FFT runs its passes in the order R3, R2, 16 and the points stay in registers from one FFT to the
-// next: 7 exchanges through shared memory instead of 9.  tw: smem_fft_chain_twiddles().
-template <int L>
-constexpr int kFftTwiddles = 16 * SmemFft<L>::R2 + (SmemFft<L>::R3 > 1 ? L : 0);
-
+// radix R leaves thread t the points t + m L/16 + r L/R (m < 16/R, r < R), which are the points t + q L/16
+// (q = m + 16/R r) of the first, radix-16 pass: they stay in registers from one FFT to the next, two
+// of the nine exchanges through shared memory fall away, and every operation and its rounding is
+// smem_fft's.
 template <int L, typename Post1, typename Post2, typename Post3>
 __device__ __forceinline__ void smem_fft_chain(float2* buf, const float2* __restrict__ tw, int t, int g, Post1&& post1,
                                                Post2&& post2, Post3&& post3) {
     using P = SmemFft<L>;
-    constexpr int T = P::T, R2 = P::R2, R3 = P::R3, RL = R3 == 1 ? R2 : R3;
-    const float2* twr = tw + kFftTwiddles<L>;
+    constexpr int T = P::T, R2 = P::R2, R3 = P::R3, RL = R3 == 1 ? R2 : R3, PER = 16 / RL;
     auto keep = [](int, float2 x) { return x; };
     float2 v[16];
-    auto exchange_done = [&] { group_sync<T>(g); };
-    // passes 16, R2, R3 up to the last one's outputs
-    auto up = [&] {
-        exchange_done();
+    // the passes after the first, up to the last one's outputs
+    auto rest = [&] {
+        group_sync<T>(g);
         gfft_store<L, 16, 1>(buf, t, v, keep);
-        exchange_done();
+        group_sync<T>(g);
         gfft_load<L, R2, 16>(buf, tw, t, v);
-        exchange_done();
+        group_sync<T>(g);
         if constexpr (R3 > 1) {
             gfft_store<L, R2, 16>(buf, t, v, keep);
-            exchange_done();
+            group_sync<T>(g);
             gfft_load<L, R3, 16 * R2>(buf, tw + 16 * R2, t, v);
-            exchange_done();
+            group_sync<T>(g);
         }
     };
+    auto next = [&](auto&& post) {
+        float2 u[16];
+#pragma unroll
+        for (int m = 0; m < PER; ++m)
+#pragma unroll
+            for (int r = 0; r < RL; ++r) u[m + PER * r] = post(t + m * T + r * (L / RL), v[m * RL + r]);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = u[q];
+        gfft_dft<L, 16, 1>(tw, t, v);
+        rest();
+    };
     gfft_load<L, 16, 1>(buf, tw, t, v);
-    up();
-#pragma unroll
-    for (int m = 0; m < 16 / RL; ++m)
-#pragma unroll
-        for (int r = 0; r < RL; ++r) v[m * RL + r] = post1(t + m * T + r * (L / RL), v[m * RL + r]);
-    gfft_dft<L, RL, 1>(tw, t, v);
-    gfft_store<L, RL, 1>(buf, t, v, keep);
-    exchange_done();
-    if constexpr (R3 > 1) {
-        gfft_load<L, R2, R3>(buf, twr, t, v);
-        exchange_done();
-        gfft_store<L, R2, R3>(buf, t, v, keep);
-        exchange_done();
-        gfft_load<L, 16, R2 * R3>(buf, twr + R2 * R3, t, v);
-    } else {
-        gfft_load<L, 16, R2>(buf, twr, t, v);
-    }
-#pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = post2(t + r * T, v[r]);
-    gfft_dft<L, 16, 1>(tw, t, v);
-    up();
+    rest();
+    next(post1);
+    next(post2);
     gfft_store<L, RL, L / RL>(buf, t, v, post3);
-    exchange_done();
+    group_sync<T>(g);
 }
 
 // the twiddle table of smem_fft<L>, from FP64 and rounded once
 std::vector<float2> smem_fft_twiddles(int L);
-// ... followed by those of the passes in the order R3, R2, 16: [R2][R3], then [16][R2 R3]
-std::vector<float2> smem_fft_chain_twiddles(int L);
 
 }  // namespace gbx
