@@ -190,8 +190,9 @@ multibeam_tc_kernel(const float* __restrict__ spec, int n_ant, int n_pol, int n_
         // ------------------------------------------------------------ MMA issuer
         // the whole warp waits and one elected lane issues: from an elect branch the products follow
         // each other at the tensor pipe's rate (N = 128: 64 clocks; from a lane == 0 branch 129 and
-        // more).  With the converters' and drains' voted waits: 32 antennas x 2, 512 channels, 2048
-        // spectra 424 -> 414 us for 32 beams and 457 -> 439 for 64, 60 inputs and 25 beams 58 -> 50.5;
+        // more).  With the converters' and drains' voted waits: 32 antennas x 2, 1024 channels, 2048
+        // spectra 424 -> 414 us for 32 beams and 457 -> 439 for 64; 60 antennas x 1, 128 channels,
+        // 2048 spectra, 25 beams 58 -> 50.5;
         // the converters bound it now.
         const uint32_t idesc = idesc_f16_f32(kRows, G.N);
         const uint32_t lbo_a = kRows * 16, lbo_b = static_cast<uint32_t>(G.N) * 16, sbo = 128;

@@ -23,13 +23,13 @@
 // thread hold a whole Gram row's running sums), warps 2, 3 and 8-15 convert the input
 // stages (96 registers).
 // What bounds the converted forms: at the GMRT shape (64 inputs, 1024 channels, 8192 spectra)
-// the FP32 form takes 0.79 ms, where its 4.3 GB alone stream in 0.61 ms, its MMAs take 0.33 ms
-// and its converters 0.54 ms, each role timed with the others idle; together they share the
+// the FP32 form takes 0.80 ms, where its 4.3 GB alone stream in 0.60 ms, its MMAs take 0.31 ms
+// and its converters 0.57 ms, each role timed with the others idle; together they share the
 // shared-memory pipe (per 64-frame stage: 32 KB landed, 32 read, 32 written, 48 of operands, and
 // the drain's TMEM reads).  It was 0.93 ms with a second MMA a step (now T + T^T, write_pair),
 // MMAs issued from a lane == 0 branch, one-lane waits and the running sums in shared memory.
-// The int8 form takes 0.36 ms (0.47 before) and is paced by its TMA gather: 16-byte pieces,
-// 0.28 ms alone.
+// The int8 form takes 0.31 ms (0.45 before) and is paced by its TMA gather of 16-byte pieces, 0.31 ms
+// alone (MMAs 0.21, converters 0.22).
 // Accumulation is chunked: every `chunk` frames the FP32 accumulator is drained
 // and added into a running sum.  Items with N <= 128 rotate over four 128-column
 // accumulators (the MMAs run up to three chunks ahead of the drain) and keep the
@@ -89,7 +89,7 @@ static_assert(kEpiThreads2 * kRegsDrain + (kWarps2 * 32 - kEpiThreads2) * kRegsO
 constexpr int kStages = 5;                    // fp16 operand slots (one-plane forms)
 constexpr int kSlot = kStageMaxBytes + 2048;  // rows past R stay in bounds
 constexpr int kTailSlack = 32768;
-// FP32 form: stages of kStage2Bytes of FP32 each, five in flight.  An operand slot takes ks * 2 n_in * 4 bytes plus the rows the
+// FP32 form: stages of kStage2Bytes of FP32 each, three in flight.  An operand slot takes ks * 2 n_in * 4 bytes plus the rows the
 // 128-row MMA reads past R; ks * rows_fp32(n_in) * 4 <= kStage2Bytes bounds that by
 // kStage2Bytes + (128 - 64) * 16 (R < 64 leaves more room).
 constexpr int kOpStages2 = 3;                 // operand slots ...
@@ -461,10 +461,9 @@ __device__ __forceinline__ void split_pair(float2 w, float2 sc, float2 nsc, floa
 // FP32 values are scaled by the power of two split_scale, hi rounded to fp16 and lo the remainder
 // rounded to fp16 (split_pair); the lo tile follows the hi tile, or in paired items (128 rows)
 // K-block j holds 128 hi rows then 128 lo rows (4096 bytes).
-// Each converter warp works on its own units and signals on its own: lane 0 waits for the slots (the
-// decision is shared by a shuffle), the warp converts, fences its shared stores for the tensor
-// core's (async) proxy, and lane 0 arrives on both slots' barriers, which complete after all
-// kConvWarps warps.  No barrier spans warps.  The body is inlined: called as a function, its
+// Each converter warp works on its own units and signals on its own: the whole warp waits for the
+// slots by vote, converts, fences its shared stores for the tensor core's (async) proxy, and
+// lane 0 arrives on both slots' barriers, which complete after all kConvWarps warps.  No barrier spans warps.  The body is inlined: called as a function, its
 // shared-memory accesses cost about twice the time.
 template <bool kIn8, bool kPairs>
 __device__ __forceinline__ void convert_stages(const XtBatch& t, Shared& sh, unsigned char* smem, int ct) {
