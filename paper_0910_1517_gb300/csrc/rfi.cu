@@ -333,7 +333,7 @@ struct Wts {
     TA* pf16;                   // [NPAR] flat
     TA *wf1, *wf2, *wf3;        // forward  [CI][9][CO]
     TA *wb3, *wb2;              // backward [CO_fwd][9][CI_fwd], taps flipped
-    unsigned char* pack;        // fp16: the tensor-core forward pass's operands (rfi_pack1 .. 3)
+    unsigned char* pack;        // fp16: the tensor-core forward pass's operands (rfi_pack2, rfi_pack3)
 };
 
 template <typename TA>
